@@ -141,11 +141,12 @@ struct Plan {
   Layout L{};
   Weights W{};
   int nshots = 0, nsrc = 0, nrec = 0, nt = 0, r = 0, T = 0, S = 0, kind = 0, acc = 0, form = 0;
-  bool c2d = false;  // 2-D batch on the persistent cluster path (tp_sweep2d_cluster.cu)
+  bool c2d = false;  // 2-D batch on the persistent path (tp_sweep2d_cluster.cu)
+  size_t o_edge = 0; // its edge words
   int comp = 0;      // compensated (double-float) forward
   size_t o_e = 0;    // comp: bf16 low parts of two levels per shot
   float scale = 1.f;
-  size_t bytes = 0;
+  size_t bytes = 0, c2_bytes = 0;
   size_t o_scal = 0, o_part = 0, o_c2 = 0, o_f = 0, o_P = 0, o_V = 0, o_Q = 0, o_d = 0, o_soff = 0, o_roff = 0,
          o_cs = 0, o_cr = 0, o_qbar = 0, o_gacc = 0, o_sacc = 0, o_conv = 0, o_w = 0;
   // deterministic injection groups of the sources and of the receivers
@@ -237,13 +238,16 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
   P->o_rshared = take(cur, (size_t)ns * P->nrec * sizeof(int));
   P->o_sn = take(cur, (size_t)ns * sizeof(int));
   P->o_rn = take(cur, (size_t)ns * sizeof(int));
-  P->o_c2 = take(cur, fb);
+  P->c2_bytes = fb + (P->L.ndim == 2 ? (size_t)8 * P->L.plane * sizeof(float) : 0);  // + rows that a 2-D band's last chunk reads
+  P->o_c2 = take(cur, P->c2_bytes);
   P->form = g->form;
   P->comp = g->form == TP_FORM_COMPENSATED;
-  P->c2d = g->form != TP_FORM_INCREMENT && cluster2d_fits(P->L, P->W, P->nshots, P->nsrc, P->nrec, P->comp);
+  P->c2d = P->comp ? cluster2d_fits(P->L, P->W, P->nshots, P->nsrc, P->nrec, true)
+                   : g->form == TP_FORM_LEVELS && persist2d_fits(P->L, P->W, P->nshots, P->nsrc, P->nrec);
   if (P->comp && !P->c2d)
     return fail(TP_ERR_ARG, "the compensated form needs a 2-D grid without an absorbing layer whose shot fits one "
                             "thread-block cluster, with at most 1024 sources and receivers per shot");
+  if (P->c2d) P->o_edge = take(cur, edge2d_bytes(P->L, P->W));
   if (P->comp) P->o_e = take(cur, (size_t)2 * ns * P->L.field * 2);  // bf16 low parts, two levels per shot
   if (P->form == TP_FORM_INCREMENT) P->o_w = take(cur, (size_t)ns * fb);  // the increment field of each shot
   switch (op) {
@@ -317,6 +321,7 @@ struct Ctx {
   const Plan& P;
   char* ws;
   cudaStream_t st;
+  mutable uint32_t tag = 1;  // persistent 2-D path: tag of the next launch's first level
   template <class T> T* at(size_t o) const { return reinterpret_cast<T*>(ws + o); }
   Scal* scal() const { return at<Scal>(P.o_scal); }
   int* err() const { return &scal()->err; }
@@ -338,7 +343,8 @@ tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float*
   const Plan& P = c.P;
   if (!vel) return fail(TP_ERR_ARG, "vel is NULL");
   TRY(cudaMemsetAsync(c.scal(), 0, SCAL_BYTES, c.st));
-  TRY(cudaMemsetAsync(c.at<float>(P.o_c2), 0, (size_t)P.L.field * sizeof(float), c.st));
+  TRY(cudaMemsetAsync(c.at<float>(P.o_c2), 0, P.c2_bytes, c.st));
+  if (P.c2d) TRY(cudaMemsetAsync(c.at<char>(P.o_edge), 0, edge2d_bytes(P.L, P.W), c.st));
   const double dt2 = (double)g->dt * (double)g->dt;
   TRY(launch_prep_c2(P.L, vel, dt2 / ((double)g->h * (double)g->h), c.at<float>(P.o_c2), c.st));
   TRY(launch_prep_points(P.L, P.W, geo->src, (long long)P.nshots * P.nsrc, vel, dt2, c.at<long long>(P.o_soff),
@@ -430,12 +436,17 @@ Cluster2dArgs cluster_args(const Ctx& c, const Fam& f, int dir, int lev0, int ns
   a.lev0 = lev0;
   a.nsteps = nsteps;
   a.fresh = fresh ? 1 : 0;
+  a.store_all = f.fs != 3;  // of a family of three levels only the newest two are read later
   a.ring = c.at<float>(f.off);
   a.nslots = f.fs;
   a.ring_ss = c.ss(f);
   a.eslots = comp ? c.at<char>(P.o_e) : nullptr;
   a.e_ss = 2 * P.L.field;
   a.c2 = c.at<float>(P.o_c2);
+  a.edge = c.at<char>(P.o_edge);
+  a.tag0 = c.tag;
+  c.tag += (uint32_t)P.nshots * (uint32_t)nsteps;
+  a.err = c.err();
   return a;
 }
 

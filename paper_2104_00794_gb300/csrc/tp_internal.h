@@ -119,33 +119,41 @@ bool encode_field_map(const Layout& L, const void* base, long long nfields, int 
                       int box_fields, CUtensorMap* out);
 
 // ---------------------------------------------------------------- 2-D cluster stepping
-// Persistent 2-D time stepping (tp_sweep2d_cluster.cu): one thread-block
-// cluster per shot holds the shot's levels in shared memory and runs nsteps
+// Persistent 2-D time stepping (tp_sweep2d_cluster.cu): bands of rows of every
+// shot, one CTA each, hold the shot's levels in shared memory and run nsteps
 // steps per launch, with in-kernel injection (entries at one node summed in
 // index order) and sampling.  Forward (dir = +1): step i forms level
 // lev0 + i + 1 from lev0 + i and lev0 + i - 1; adjoint (dir = -1): level
-// lev0 - i - 1 from lev0 - i and lev0 - i + 1.  Every new level is written to
-// ring slot (level mod nslots) of its shot; the launch starts from the ring
-// slots of lev0 and lev0 - dir (zero when fresh).  comp: double-float levels
-// (low parts in bf16 slots eslots + shot * e_ss + (level mod 2) * field,
-// written for the last two levels of a launch).  Injection: new level at
+// lev0 - i - 1 from lev0 - i and lev0 - i + 1.  Every new level (store_all), or
+// the last two, is written to ring slot (level mod nslots) of its shot; the
+// launch starts from the ring slots of lev0 and lev0 - dir (zero when fresh).
+// comp: double-float levels (low parts in bf16 slots eslots + shot * e_ss +
+// (level mod 2) * field, written for the last two levels of a launch).  An
+// absorbing layer (W.sw) is stepped in the levels form.  Injection: new level at
 // inj_off[s][k] += inj_coef[s][k] * inj_val[s][new level + inj_shift][k];
 // sampling: samp_out[s][new level + samp_shift][j] = new level at samp_off[s][j].
+// edge: edge2d_bytes() of scratch, zeroed before the first launch that uses it;
+// tag0 >= 1, raised by nshots * nsteps from launch to launch.
 struct Cluster2dArgs {
   Layout L;
   Weights W;
-  int nshots, comp, dir, lev0, nsteps, fresh;
+  int nshots, comp, dir, lev0, nsteps, fresh, store_all;
   float* ring; int nslots; long long ring_ss;
   void* eslots; long long e_ss;
   const float* c2;
   const long long* inj_off; const float* inj_coef; int ninj;
   const float* inj_val; long long inj_val_ss; int inj_shift;
   const long long* samp_off; int nsamp; float* samp_out; long long samp_out_ss; int samp_shift;
+  void* edge; uint32_t tag0; int* err;
 };
 cudaError_t launch_cluster2d(const Cluster2dArgs& a, cudaStream_t s);
-// whether the cluster path can run a batch of this grid (2-D, no absorbing
-// layer, a shot's bands fit one cluster, at most 1024 sources and receivers)
+// whether a shot of this grid fits one thread-block cluster (2-D, no absorbing
+// layer, at most 1024 sources and receivers): the compensated form's condition
 bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec, bool comp);
+// whether the levels form (with or without an absorbing layer) can run on
+// bands of the whole GPU
+bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec);
+size_t edge2d_bytes(const Layout& L, const Weights& W);
 
 // ---------------------------------------------------------------- probe GEMM
 // P[s][i][x] += sum_{k < nlev} ring[s][(level0 + k) mod nslots][x] * Q[s][level0 + k + qshift][i]

@@ -1,44 +1,59 @@
-// Persistent 2-D time stepping on thread-block clusters (sm_103a).
+// Persistent 2-D time stepping (sm_103a): a shot's rows are split into bands,
+// one CTA per band, and every launch runs many time steps.
 //
-// Algorithm 1 lines 1 and 5 (operators f and f^T) for a batch of 2-D shots,
-// many time steps per launch.  A 2-D shot is small (801 x 301 points: 1 MB
-// per level), so one cluster of up to 16 CTAs holds a whole shot's state in
-// shared memory and steps it without a round trip through L2 or a kernel
-// launch per step:
-//   * CTA k of a cluster owns a band of rpc grid rows.  Its shared memory
-//     holds the band of the current and the previous level (ping-pong: the
-//     new level overwrites the previous one point by point), rows of
-//     4 + nx + 4 floats with zero columns for the x stencil;
-//   * z neighbours beyond the band are read from the neighbouring CTAs'
-//     shared memory (distributed shared memory, generic loads through
-//     cluster-mapped addresses), rows outside the grid from a zero row;
-//   * one step is: compute the band's new level (results kept in registers
-//     until every load of the step is issued), __syncthreads, add the
-//     sources of the step (one thread per distinct node, entries at a node
-//     summed in index order: deterministic), one cluster barrier;
-//   * every level is also copied to its slot of a ring in global memory (the
-//     window GEMM of the probe accumulation reads it, and the next launch
-//     restarts from it) by asynchronous bulk copies of its rows, issued when
-//     the next step starts: the cluster barrier's release would wait for
-//     plain global stores, not for these; its receivers are sampled from
-//     shared memory;
-//   * each thread owns a float4 column of a chunk of the band's rows for the
-//     whole launch and marches down it with the z neighbours in a register
-//     queue (c2 comes through the read-only cache); rows of the band are read
-//     by shared-memory address, rows of other bands through a table of
-//     cluster-mapped row addresses;
-//   * the cluster size is chosen per grid and device: the least work per CTA
-//     over the rounds of clusters the batch needs (at most 16 CTAs).
+// Algorithm 1 lines 1 and 5 (operators f and f^T) for a batch of 2-D shots.
+// A 2-D shot is small (801 x 301 points: 1 MB per level), so its state stays
+// in shared memory and is stepped without a kernel launch per step:
+//   * CTA k of a shot owns a band of rpc grid rows.  Its shared memory holds
+//     the band of the current and the previous level (ping-pong: the new level
+//     overwrites the previous one point by point), rows of 4 + nx + 4 floats
+//     with zero columns for the x stencil, and c2 where it fits;
+//   * a thread marches along one float4 column of a chunk of N rows, the z
+//     neighbours in a register queue.  N is a template parameter and the band a
+//     whole number of chunks, so that no row and no column is guarded (rows past
+//     the grid and columns past nx have c2 = 0 and stay zero): with a guarded
+//     loop a step took 237 warp instructions per 128 points, now 145, of which
+//     the stencil needs 66;
+//   * the first and the last chunk march away from the neighbouring bands, so
+//     the rows that a neighbour needs are formed first;
+//   * entries that inject at a node are added by the thread that owns the
+//     node, in index order (deterministic);
+//   * the levels that the caller needs go to their ring slots in global memory
+//     (the window GEMM reads them, the next launch starts from them).
+// Two exchanges of the band edges (the R rows next to a neighbour):
+//   * cluster: the bands of a shot are one thread-block cluster (at most 16
+//     CTAs); edges are read from the neighbour's shared memory, one cluster
+//     barrier per step (470 cycles);
+//   * bands (BAND): the bands of all shots of the batch are one cooperative
+//     grid over the whole GPU.  A thread stores the edge values it forms also
+//     as 8-byte words (value, step tag) in global memory; the neighbour's
+//     thread of the same column, the only one that needs them, loads the words
+//     when its march ends and reads again as the next one begins until they
+//     carry the step's tag: no fence and no flag (1640-2480 cycles from the store
+//     to the reader; 3100 for a flag behind a fence), and most of that passes
+//     while the rest of the band is marched.  The wait is bounded: on a timeout
+//     the CTA sets bit 0 of *err and steps on without waiting (its results are
+//     then invalid).
+// Why both: clusters of this size leave SMs idle (8 shots of 12 CTAs: 96 of
+// 152 SMs; 7 clusters of 16 at once), bands use all of them, but an exchange
+// through L2 costs more than a cluster barrier, which decides on small grids;
+// c2_step_cost has the measurements.
+// Measured per step on GB300, before (clusters only, one CTA of 16 warps with
+// guarded rows) and now: 601 x 201, 16 shots, order 8: levels 6.8 -> 3.9 us,
+// compensated 12.6 -> 8.1 us; 801 x 301, 8 shots: 7.1 -> 3.9, 18.6 -> 8.0 us; 101
+// x 101, one shot, order 4: 2.0 -> 1.5 us; an absorbing layer (601 x 201, 4
+// shots, then two launches per step) 29 -> 4.6 us.  Bound by the shared memory
+// pipe (32 wavefronts per 128 points of the levels form: the row and its
+// neighbours, c2, the previous and the new level, the ring) and by issue.
+//
 // Levels form: the arithmetic of the per-step 2-D sweep, operation for
-// operation (bit-identical results).  Compensated form (forward only): the
-// wavefield is a double-float u + e (e stored as bf16) stepped with an
-// error-free transformation, so that the rounding of the stored levels, which
-// the Laplacian of the probed field amplifies, is carried instead of lost;
-// the Laplacian of u is taken in the per-neighbour difference form, exact for
-// neighbours within a factor of two of the centre.
-// The kernel has no spin-waits: its only waits are hardware barriers that
-// every thread of the cluster reaches the same number of times.
-#include <cooperative_groups.h>
+// operation (bit-identical results), with or without the absorbing layer.
+// Compensated form (forward only): the wavefield is a double-float u + e (e
+// stored as bf16) stepped with an error-free transformation, so that the
+// rounding of the stored levels, which the Laplacian of the probed field
+// amplifies, is carried instead of lost; the Laplacian of u is taken in the
+// per-neighbour difference form, exact for neighbours within a factor of two of
+// the centre.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -46,8 +61,6 @@
 #include <vector>
 
 #include "tp_internal.h"
-
-namespace cg = cooperative_groups;
 
 namespace tp {
 
@@ -57,14 +70,16 @@ constexpr int C2_THREADS = 512;
 constexpr int C2_MAXCOL = C2_THREADS;  // float4 columns of a band (nx <= 2048)
 constexpr int C2_MAXLIST = 1024; // injection or sampling entries of one shot
 constexpr int C2_MAXC = 16;      // cluster size limit (non-portable above 8)
-constexpr int C2_PER = C2_MAXLIST / C2_THREADS;  // list entries per thread
+constexpr int C2_MAXBANDS = 152; // CTAs of a cooperative launch
+constexpr size_t C2_SMEM = 227 * 1024;
 
+enum C2Mode { C2_LEVELS = 0, C2_COMP = 1, C2_DAMP = 2 };
 struct C2Args {
   Layout L;
   Weights W;
   int nshots, C, rpc, sx, nx4;
   int capi, caps;  // capacities of a band's injection and sampling lists (entries)
-  int comp, dir, lev0, nsteps, fresh;
+  int dir, lev0, nsteps, fresh, store_all;
   float* ring; int nslots; long long ring_ss;  // level l of shot s: ring + s*ring_ss + (l % nslots)*L.field
   __nv_bfloat16* eslots; long long e_ss;       // comp: e of level l: eslots + s*e_ss + (l % 2)*L.field
   const float* c2;
@@ -72,26 +87,22 @@ struct C2Args {
   const float* inj_val; long long inj_val_ss; int inj_shift;   // row of the values: new level + inj_shift
   const long long* samp_off; int nsamp;
   float* samp_out; long long samp_out_ss; int samp_shift;      // row of the output: new level + samp_shift
+  unsigned char* edge;  // BAND: tagged edge words, [plane][cta][side][parity][row][column] of 16 bytes
+  uint32_t tag0;        // tag of level lev0 in the first round of shots
+  long long spin;       // limit of a wait for an edge word (cycles)
+  int* err;
 };
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
-// bf16 <-> fp32 helpers for four values
-__device__ __forceinline__ float4 ld_bf4(const __nv_bfloat16* p) {
-  const uint2 r = *reinterpret_cast<const uint2*>(p);
-  float4 v;
-  v.x = __uint_as_float(r.x << 16);
-  v.y = __uint_as_float(r.x & 0xffff0000u);
-  v.z = __uint_as_float(r.y << 16);
-  v.w = __uint_as_float(r.y & 0xffff0000u);
-  return v;
+// bf16 <-> fp32 for four values
+__device__ __forceinline__ float4 bf4(uint2 r) {
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                     __uint_as_float(r.y & 0xffff0000u));
 }
-__device__ __forceinline__ void st_bf4(__nv_bfloat16* p, float4 v) {
+__device__ __forceinline__ uint2 to_bf4(float4 v) {
   const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-  uint2 r;
-  r.x = *reinterpret_cast<const uint32_t*>(&a);
-  r.y = *reinterpret_cast<const uint32_t*>(&b);
-  *reinterpret_cast<uint2*>(p) = r;
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
 }
 
 // s = a + b exactly as s + err (Knuth's TwoSum, 6 operations)
@@ -102,21 +113,7 @@ __device__ __forceinline__ float two_sum(float a, float b, float* err) {
   return s;
 }
 
-// one row of a band (shared memory) to its place in a global field, as an
-// asynchronous bulk copy: the cluster barrier's release does not wait for it
-__device__ __forceinline__ void bulk_row_store(float* gdst, const float* ssrc, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
-               "r"((uint32_t)__cvta_generic_to_shared(ssrc)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// the bulk copies of this thread have read their shared memory sources
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// ... and have completed
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// generic-proxy writes to shared memory become visible to the bulk copies
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-
+__device__ __forceinline__ uint32_t sa(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ float4 lds4(uint32_t a) {
   float4 v;
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
@@ -127,90 +124,321 @@ __device__ __forceinline__ uint2 lds2(uint32_t a) {
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
   return v;
 }
-__device__ __forceinline__ float4 bf4(uint2 r) {
-  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
-                     __uint_as_float(r.y & 0xffff0000u));
+__device__ __forceinline__ int ldsi(uint32_t a) {
+  int v;
+  asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ int4 ldsi4(uint32_t a) {
+  int4 v;
+  asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void sts2(uint32_t a, uint2 v) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+// the same from any CTA of the cluster (shared::cluster address)
+__device__ __forceinline__ float4 ldc4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 ldc2(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t a, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// Two edge words of 8 bytes, each a 32-bit value and the tag of its step; a
+// word is written and read as one access, so a fresh tag brings its value.
+__device__ __forceinline__ uint4 ld_words(const unsigned char* p) {
+  unsigned long long a, b;
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p));
+  return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+}
+__device__ __forceinline__ void st_words(unsigned char* p, uint32_t v0, uint32_t v1, uint32_t tag) {
+  const unsigned long long a = ((unsigned long long)tag << 32) | v0, b = ((unsigned long long)tag << 32) | v1;
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
 
 __device__ __forceinline__ float comp4(const float4& v, int p) {
   return p == 0 ? v.x : (p == 1 ? v.y : (p == 2 ? v.z : v.w));
 }
 
-template <int R, bool COMP>
-__global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_cluster(C2Args a) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int ncl = gridDim.x / a.C, cid = blockIdx.x / a.C;
+// n / b, b = 1 + a of the absorbing layer, with inv = 1 / b correctly rounded:
+// two residual corrections give the correctly rounded quotient (Markstein 1990)
+// while the residual does not underflow.  The values ahead of a wave are tiny
+// over most of a layer; they are divided scaled by 2^96, and a subnormal result,
+// then rounded a second time, moves to its other neighbour where the first
+// rounding had made a tie.  (A plain division, with its slow branch for zeros and
+// tiny values, took 13 us of a 17 us step: 601 x 201, 16 shots.)
+__device__ __forceinline__ float quotient(float n, float b, float inv) {
+  const bool tiny = fabsf(n) < 0x1p-60f;
+  if (tiny) n *= 0x1p96f;
+  float q = n * inv;
+  q = fmaf(fmaf(-q, b, n), inv, q);
+  const float r = fmaf(-q, b, n);
+  q = fmaf(r, inv, q);
+  if (tiny) {
+    const float s = q, d = s * 0x1p-96f, diff = fmaf(d, -0x1p96f, s);
+    q = d;
+    if (fabsf(diff) == 0x1p-54f && fmaf(-s, b, n) * diff > 0.f) q += copysignf(0x1p-149f, diff);
+  }
+  return fabsf(n) <= 3.402823466e38f ? q : n;  // infinities and NaN: no residual
+}
+
+// The operators of one row, 4 points: u[i] the rows i - R of the column (u[R]
+// the row itself), low(k) the low parts of row k of the column (COMP; 0: the row
+// itself), cq = c2; in shared memory the row (ua, for the neighbours in x) and
+// the previous level (na), low parts at eoff and neff + address / 2.  o: the new level,
+// en: its low part; c1, s2: the previous level and the sums of S(u) (for the
+// absorbing layer).
+template <int R, int MODE, class Low>
+__device__ __forceinline__ void row4(const Weights& W, const float4* u, Low low, float4 cq, uint32_t ua, uint32_t na,
+                                     uint32_t eoff, uint32_t neff, float (&o)[4], float (&en)[4], float4& c1,
+                                     float2 (&s2)[2]) {
+  constexpr bool COMP = MODE == C2_COMP;
+  const float2 m4 = f2(-4.f, -4.f), m1 = f2(-1.f, -1.f), two = f2(2.f, 2.f);
+  const float4 xc = u[R];
+  if (!COMP) {
+    const float4 xl = lds4(ua - 16u), xr = lds4(ua + 16u);
+    const float v[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w, xr.x, xr.y, xr.z, xr.w};
+    c1 = lds4(na);
+    // centred form, the per-step 2-D sweep's operations in its order (two
+    // points per packed instruction; the x pairs at odd distances are not
+    // register pairs, so those sums are scalar)
+#pragma unroll
+    for (int k = 1; k <= R; ++k) {
+      const float4 zp = u[R + k], zm = u[R - k];
+      const float2 wk = f2(W.w[k], W.w[k]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int pp = 2 * h;
+        const float2 xs = (k & 1) ? f2(__fadd_rn(v[4 + pp + k], v[4 + pp - k]), __fadd_rn(v[5 + pp + k], v[5 + pp - k]))
+                                  : __fadd2_rn(f2(v[4 + pp + k], v[5 + pp + k]), f2(v[4 + pp - k], v[5 + pp - k]));
+        const float2 zs = __fadd2_rn(h ? f2(zp.z, zp.w) : f2(zp.x, zp.y), h ? f2(zm.z, zm.w) : f2(zm.x, zm.y));
+        const float2 t = __ffma2_rn(m4, f2(v[4 + pp], v[5 + pp]), __fadd2_rn(xs, zs));
+        s2[h] = k == 1 ? __fmul2_rn(wk, t) : __ffma2_rn(wk, t, s2[h]);
+      }
+    }
+    // new = c2 S + (2u - u_prev); 2u is exact, so the FMA rounds 2u - u_prev once, as a subtraction
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      o[p] = fmaf(comp4(cq, p), p & 1 ? s2[p / 2].y : s2[p / 2].x, fmaf(2.f, v[4 + p], -comp4(c1, p)));
+    return;
+  }
+  // double-float levels: U = u + e.  S(e) in the centred form (e is a few ulp of
+  // u: its rounding is negligible), S(u) in the difference form for k = 1, 2 and
+  // the centred form for the small weights k = 3, 4 (their rounding is a few
+  // hundredths of an ulp of u)
+  const uint32_t ea = eoff + ua / 2u;
+  const float4 fl = bf4(lds2(ea - 8u)), fr = bf4(lds2(ea + 8u)), fc = bf4(low(0));
+  const float ve[12] = {fl.x, fl.y, fl.z, fl.w, fc.x, fc.y, fc.z, fc.w, fr.x, fr.y, fr.z, fr.w};
+  float2 su[2], se[2];
+#pragma unroll
+  for (int k = 1; k <= R; ++k) {
+    const float4 ezp = bf4(low(k)), ezm = bf4(low(-k));
+    const float2 wk = f2(W.w[k], W.w[k]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int pp = 2 * h;
+      const float2 xe = (k & 1) ? f2(__fadd_rn(ve[4 + pp + k], ve[4 + pp - k]), __fadd_rn(ve[5 + pp + k], ve[5 + pp - k]))
+                                : __fadd2_rn(f2(ve[4 + pp + k], ve[5 + pp + k]), f2(ve[4 + pp - k], ve[5 + pp - k]));
+      const float2 ze = __fadd2_rn(h ? f2(ezp.z, ezp.w) : f2(ezp.x, ezp.y), h ? f2(ezm.z, ezm.w) : f2(ezm.x, ezm.y));
+      const float2 te = __ffma2_rn(m4, f2(ve[4 + pp], ve[5 + pp]), __fadd2_rn(xe, ze));
+      se[h] = k == 1 ? __fmul2_rn(wk, te) : __ffma2_rn(wk, te, se[h]);
+    }
+  }
+  const float4 xl = lds4(ua - 16u), xr = lds4(ua + 16u);
+  const float v[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w, xr.x, xr.y, xr.z, xr.w};
+#pragma unroll
+  for (int k = 1; k <= R; ++k) {
+    const float4 zp = u[R + k], zm = u[R - k];
+    const float2 wk = f2(W.w[k], W.w[k]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int pp = 2 * h;
+      const float2 cv = f2(v[4 + pp], v[5 + pp]);
+      const float2 zpp = h ? f2(zp.z, zp.w) : f2(zp.x, zp.y), zmm = h ? f2(zm.z, zm.w) : f2(zm.x, zm.y);
+      float2 t;
+      if (k <= 2) {
+        // the two heavy weights: per-neighbour differences, exact for
+        // neighbours within a factor two of the centre
+        float2 dxp, dxm;
+        if (k & 1) {
+          dxp = f2(__fadd_rn(v[4 + pp + k], -cv.x), __fadd_rn(v[5 + pp + k], -cv.y));
+          dxm = f2(__fadd_rn(v[4 + pp - k], -cv.x), __fadd_rn(v[5 + pp - k], -cv.y));
+        } else {
+          dxp = __ffma2_rn(m1, cv, f2(v[4 + pp + k], v[5 + pp + k]));
+          dxm = __ffma2_rn(m1, cv, f2(v[4 + pp - k], v[5 + pp - k]));
+        }
+        const float2 dzp = __ffma2_rn(m1, cv, zpp), dzm = __ffma2_rn(m1, cv, zmm);
+        t = __fadd2_rn(__fadd2_rn(dxp, dxm), __fadd2_rn(dzp, dzm));
+      } else {
+        const float2 xs = (k & 1) ? f2(__fadd_rn(v[4 + pp + k], v[4 + pp - k]), __fadd_rn(v[5 + pp + k], v[5 + pp - k]))
+                                  : __fadd2_rn(f2(v[4 + pp + k], v[5 + pp + k]), f2(v[4 + pp - k], v[5 + pp - k]));
+        t = __ffma2_rn(m4, cv, __fadd2_rn(xs, __fadd2_rn(zpp, zmm)));
+      }
+      su[h] = k == 1 ? __fmul2_rn(wk, t) : __ffma2_rn(wk, t, su[h]);
+    }
+  }
+  c1 = lds4(na);
+  const float4 f1 = bf4(lds2(neff + na / 2u));
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int pp = 2 * h;
+    const float2 uu = f2(v[4 + pp], v[5 + pp]), ee = f2(ve[4 + pp], ve[5 + pp]);
+    const float2 cp = f2(comp4(c1, pp), comp4(c1, pp + 1)), ep = f2(comp4(f1, pp), comp4(f1, pp + 1));
+    const float2 cc2 = f2(comp4(cq, pp), comp4(cq, pp + 1));
+    // 2u - u_prev exactly (TwoSum), then the small terms, then TwoSum again
+    // (x - y as fma(-1, y, x): the product is exact)
+    const float2 u2 = __fmul2_rn(two, uu);
+    const float2 av = __ffma2_rn(m1, cp, u2);
+    const float2 bb = __ffma2_rn(m1, u2, av);
+    const float2 ea = __ffma2_rn(m1, __fadd2_rn(cp, bb), __ffma2_rn(m1, __ffma2_rn(m1, bb, av), u2));
+    const float2 b = __ffma2_rn(cc2, __fadd2_rn(su[h], se[h]), __ffma2_rn(m1, ep, __fmul2_rn(two, ee)));
+    const float2 bt = __fadd2_rn(b, ea);
+    const float2 sm = __fadd2_rn(av, bt);
+    const float2 b2 = __ffma2_rn(m1, av, sm);
+    const float2 er2 = __fadd2_rn(__ffma2_rn(m1, __ffma2_rn(m1, b2, sm), av), __ffma2_rn(m1, b2, bt));
+    o[pp] = sm.x;
+    o[pp + 1] = sm.y;
+    en[pp] = er2.x;
+    en[pp + 1] = er2.y;
+  }
+}
+
+// A unit of work: one float4 column of a chunk of N rows of the band, marched
+// by one thread with the z neighbours in a register queue (blocks of BL rows
+// unrolled, so that the queue moves once per block).  The band's rpc rows are a
+// multiple of N; rows past the grid and columns past nx have c2 = 0 and stay
+// zero, so that no row and no column is guarded.
+template <int R, int MODE, bool BAND, int N, bool C2S>
+__global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
+  constexpr bool COMP = MODE == C2_COMP, DAMP = MODE == C2_DAMP;
+  constexpr int PER = C2_MAXLIST / C2_THREADS;  // list entries per thread
   const int tid = threadIdx.x;
+  const int C = a.C, rank = blockIdx.x % C, cid = blockIdx.x / C, ncl = gridDim.x / C;
   const int sx = a.sx, sx4 = a.sx / 4, rpc = a.rpc, nx4 = a.nx4;
   const int nz = a.L.nz, nx = a.L.nx, px = a.L.px;
   const int z0 = rank * rpc;
-  const int nrow = max(0, min(rpc, nz - z0));  // rows this CTA owns
+  const int nrow = min(rpc, nz - z0);  // rows of the grid that this CTA owns (>= 1)
+  const int nch = rpc / N, units = nch * nx4;
 
-  // shared memory: both levels of the band, a zero row, the low parts (COMP),
-  // row tables, and the band's injection and sampling entries
+  // shared memory: both levels of the band, a zero row (clusters), the low
+  // parts of both levels (COMP), c2, the band's injection and sampling
+  // entries, the damping by distance (DAMP)
   extern __shared__ __align__(16) unsigned char smem[];
   float* const U0 = reinterpret_cast<float*>(smem);
   float* const U1 = U0 + (size_t)rpc * sx;
   float* const Z = U1 + (size_t)rpc * sx;  // zeros (as fp32 and as bf16)
-  unsigned char* p = reinterpret_cast<unsigned char*>(Z + sx);
-  __nv_bfloat16* const E0 = COMP ? reinterpret_cast<__nv_bfloat16*>(p) : nullptr;
-  __nv_bfloat16* const E1 = COMP ? E0 + (size_t)rpc * sx : nullptr;
-  if (COMP) p = reinterpret_cast<unsigned char*>(E1 + (size_t)rpc * sx);
-  const int nrt = rpc + 2 * R;
-  const float** rowU = reinterpret_cast<const float**>(p);  // [2][nrt]: rows z0 - R .. z0 + rpc + R - 1
-  const __nv_bfloat16** rowE = reinterpret_cast<const __nv_bfloat16**>(rowU + 2 * nrt);
-  int* iloc = reinterpret_cast<int*>(rowE + 2 * nrt);  // injection: node (band index)
-  int* imeta = iloc + a.capi;                           // k | leader << 16 | (next + 1) << 17
-  float* ival = reinterpret_cast<float*>(imeta + a.capi);
-  int* sloc = reinterpret_cast<int*>(ival + a.capi);    // sampling: node, column
-  int* sk = sloc + a.caps;
-  int* cnt = sk + a.caps;  // [0] injection, [1] sampling entries, [4 ..] per-warp counts
+  float* pf = Z + (BAND ? 0 : sx);
+  // bands: the low parts have R rows before and after the band (behind a
+  // march's first row), one region between the buffers for both of them
+  const int er = BAND ? R : 0;
+  __nv_bfloat16* const E0 = reinterpret_cast<__nv_bfloat16*>(pf) + (size_t)er * sx;
+  __nv_bfloat16* const E1 = E0 + (size_t)(rpc + er) * sx;
+  if (COMP) pf = reinterpret_cast<float*>(E1 + (size_t)(rpc + er) * sx);
+  float* const c2b = pf;
+  if (C2S) pf += (size_t)rpc * 4 * nx4;
+  uint32_t* const il = reinterpret_cast<uint32_t*>(pf);  // injection: node (band index) << 16 | k
+  uint32_t* const sl = il + a.capi;                      // sampling: the same
+  const int vstep = a.capi + 4;                               // floats from one step's values to the next step's
+  float* const ival = reinterpret_cast<float*>(sl + a.caps);  // [2][vstep]: values of this step and the next, [capi]: 0
+  // entries by unit: in the common case (one row of the unit, one entry per
+  // point at most) the row's place in the march and the entry of each of its 4
+  // points; else a chain of entries in index order
+  // Per unit, read where it is used (kept in registers, it spilled):
+  //   ua[u]: byte offset of its first row in a level buffer, offset in a field,
+  //          byte offset in c2, flags | its first row << 8
+  //   ub[u]: words of its first row and of the nearest row behind it (byte
+  //          offsets for parity 0), chain's first entry | march row of the line
+  //          << 16, column
+  int4* const ua_ = reinterpret_cast<int4*>(ival + 2 * vstep);
+  int4* const ub_ = ua_ + units;
+  ushort4* const uline = reinterpret_cast<ushort4*>(ub_ + units);
+  uint16_t* const tl = reinterpret_cast<uint16_t*>(uline + units);  // last entry of a unit (set-up)
+  uint16_t* const nxt = tl + (units + 1) / 2 * 2;                // next entry of the same unit
+  int* const cnt = reinterpret_cast<int*>(nxt + (units + 1) / 2 % 2 * 2 + a.capi);  // [0] injection, [1] sampling entries, [4 ..] per-warp counts
+  volatile int* const aborted = cnt + 2;
+  uint32_t* const tab = reinterpret_cast<uint32_t*>(cnt + 4 + C2_THREADS / 32);  // clusters: edge rows of the levels, low parts
+  float2* const dmp = reinterpret_cast<float2*>(tab + (BAND ? 0 : 8 * R));
+  constexpr uint32_t NONE = 0xffff;
+  constexpr int F_ON = 1, F_UP = 2, F_FULL = 4, F_NB = 8, F_OUT = 16, F_PUB = 32, F_LATE = 64;  // flags of a unit
 
-  for (int i = tid; i < 2 * nrt; i += C2_THREADS) {
-    const int b = i / nrt, zz = z0 - R + i % nrt;
-    const float* pu = Z + 4;
-    const __nv_bfloat16* pe = reinterpret_cast<const __nv_bfloat16*>(Z) + 4;
-    if (zz >= 0 && zz < nz) {
-      const int rk = zz / rpc, lr = zz - rk * rpc;
-      float* bu = (b ? U1 : U0) + (size_t)lr * sx + 4;
-      pu = rk == rank ? bu : cluster.map_shared_rank(bu, rk);
-      if (COMP) {
-        __nv_bfloat16* be = (b ? E1 : E0) + (size_t)lr * sx + 4;
-        pe = rk == rank ? be : cluster.map_shared_rank(be, rk);
+  if (!BAND) {
+    // tab[b * 2R + i] (and 4R + ...: low parts): edge row i of buffer b, rows
+    // -R .. -1 of the band, then rpc .. rpc + R - 1
+    for (int i = tid; i < 4 * R; i += C2_THREADS) {
+      const int b = i / (2 * R), e = i % (2 * R), zz = z0 + (e < R ? e - R : rpc + e - R);
+      uint32_t u = mapa(sa(Z), rank), lo = u;
+      if (zz >= 0 && zz < nz) {
+        const int rk = zz / rpc, lr = zz - rk * rpc;
+        u = mapa(sa((b ? U1 : U0) + (size_t)lr * sx), rk);
+        if (COMP) lo = mapa(sa((b ? E1 : E0) + (size_t)lr * sx), rk);
       }
+      tab[i] = u;
+      tab[4 * R + i] = lo;
     }
-    rowU[i] = pu;
-    rowE[i] = pe;
+    for (int i = tid; i < sx; i += C2_THREADS) Z[i] = 0.f;
   }
-  for (int i = tid; i < sx; i += C2_THREADS) Z[i] = 0.f;
-  // this thread's points: one float4 column cu of the band, rows [ra, rb);
-  // the band's columns are split into nchunk row chunks of hc rows
-  const int nchunk = max(1, C2_THREADS / nx4);
-  const int hc = (nrow + nchunk - 1) / max(nchunk, 1);
-  const int cu = tid % nx4, ch = tid / nx4;
-  const int ra = ch < nchunk ? min(nrow, ch * hc) : nrow;
-  const int rb = ch < nchunk ? min(nrow, ra + hc) : nrow;
-  const uint32_t sU0 = (uint32_t)__cvta_generic_to_shared(U0), sU1 = (uint32_t)__cvta_generic_to_shared(U1);
-  const uint32_t sE0 = COMP ? (uint32_t)__cvta_generic_to_shared(E0) : 0u;
-  const uint32_t sE1 = COMP ? (uint32_t)__cvta_generic_to_shared(E1) : 0u;
+  if (DAMP)  // a = samax ((sw - d) / sw)^2 by distance (sponge_a's operations) and 1 / (1 + a); [sw]: outside the layer
+    for (int d = tid; d <= a.W.sw; d += C2_THREADS) {
+      const float t = (float)(a.W.sw - d) / (float)a.W.sw, ad = a.W.samax * t * t;
+      dmp[d] = make_float2(ad, 1.0f / (1.0f + ad));
+    }
+  if (tid == 0) *aborted = 0;
+  if (C2S)
+    for (int i = tid; i < rpc * nx4; i += C2_THREADS)
+      reinterpret_cast<float4*>(c2b)[i] =
+          i / nx4 < nrow ? __ldg(reinterpret_cast<const float4*>(a.c2 + (long long)(z0 + i / nx4 + H) * px + HX) + i % nx4)
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
 
-  const float2 m4 = f2(-4.f, -4.f);
-  for (int shot = cid; shot < a.nshots; shot += ncl) {
+  const uint32_t sU0 = sa(U0), sE0 = sa(E0), sC2 = sa(c2b), lbytes = (uint32_t)(rpc * sx) * 4u;
+  const uint32_t ebytes = (uint32_t)((rpc + er) * sx) * 2u;  // from one buffer of low parts to the other
+  // chunk -> first row and direction of its march: the last chunk up, the
+  // others down, so that the rows next to a neighbour come first
+  auto march = [&](int ch, int& start, int& d) {
+    const bool up = ch > 0 && ch == nch - 1;
+    d = up ? -1 : 1;
+    start = up ? ch * N + N - 1 : ch * N;
+  };
+  // BAND: edge words, offset of (cta, side 0 first / 1 last rows, parity, row, column), planes apart
+  const uint32_t erow = (uint32_t)nx4 * 16u, epar = erow * R, eplane = gridDim.x * 4u * epar;
+  const uint32_t mine = blockIdx.x * 4u * epar;  // this CTA's words; the band above's precede them, below's follow
+  auto publish = [&](uint32_t o, float4 v, uint2 e, uint32_t tag) {
+    unsigned char* w = a.edge + o;
+    st_words(w, __float_as_uint(v.x), __float_as_uint(v.y), tag);
+    st_words(w + eplane, __float_as_uint(v.z), __float_as_uint(v.w), tag);
+    if (COMP) st_words(w + 2 * eplane, e.x, e.y, tag);
+  };
+
+  uint32_t tagb = a.tag0;
+  for (int shot = cid; shot < a.nshots; shot += ncl, tagb += (uint32_t)a.nsteps) {
     // ---------------------------------------------------------- per-shot set-up
     // this band's injection and sampling entries, compacted in index order
     for (int list = 0; list < 2; ++list) {
-      const int n = list == 0 ? a.ninj : a.nsamp;
+      const int num = list == 0 ? a.ninj : a.nsamp;
       const long long* off = list == 0 ? a.inj_off + (long long)shot * a.ninj
-                                       : (n > 0 ? a.samp_off + (long long)shot * a.nsamp : nullptr);
-      int* loc = list == 0 ? iloc : sloc;
-      int* kk = list == 0 ? imeta : sk;
+                                       : (num > 0 ? a.samp_off + (long long)shot * a.nsamp : nullptr);
+      uint32_t* out = list == 0 ? il : sl;
       if (tid == 0) cnt[list] = 0;
       __syncthreads();
-      for (int base = 0; base < n; base += C2_THREADS) {
+      for (int base = 0; base < num; base += C2_THREADS) {
         const int k = base + tid;
         int l = -1;
-        if (k < n) {
+        if (k < num) {
           const long long o = off[k];
           if (o >= 0) {
             const int zz = (int)(o / px) - H, xx = (int)(o % px) - HX;
@@ -222,11 +450,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_cluster(C2Args a) {
         __syncthreads();
         int before = 0;
         for (int w = 0; w < (tid >> 5); ++w) before += cnt[4 + w];
-        if (l >= 0) {
-          const int pos = cnt[list] + before + __popc(m & ((1u << (tid & 31)) - 1u));
-          loc[pos] = l;
-          kk[pos] = k;
-        }
+        if (l >= 0) out[cnt[list] + before + __popc(m & ((1u << (tid & 31)) - 1u))] = (uint32_t)l << 16 | (uint32_t)k;
         __syncthreads();
         if (tid == 0) {
           int tot = 0;
@@ -237,321 +461,521 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_cluster(C2Args a) {
       }
     }
     const int ni = cnt[0], ns = cnt[1];
-    // coincident injection points: the first entry at a node leads, the
-    // others follow it in index order
-    float pc[C2_PER];
-    int pk[C2_PER];
-#pragma unroll
-    for (int q = 0; q < C2_PER; ++q) {
-      const int i = tid + q * C2_THREADS;
-      pc[q] = 0.f;
-      pk[q] = 0;
-      if (i < ni) {
-        int nxt = -1;
-        for (int j = i + 1; j < ni; ++j)
-          if (iloc[j] == iloc[i]) { nxt = j; break; }
-        bool lead = true;
-        for (int j = 0; j < i; ++j)
-          if (iloc[j] == iloc[i]) { lead = false; break; }
-        pk[q] = imeta[i];
-        pc[q] = a.inj_coef[(long long)shot * a.ninj + pk[q]];
-        imeta[i] = pk[q] | (lead ? 1 << 16 : 0) | ((nxt + 1) << 17);
+    // a chain of entries per unit, in index order
+    for (int u = tid; u < units; u += C2_THREADS) {
+      ub_[u].z = (int)(NONE << 16 | NONE);
+      tl[u] = (uint16_t)NONE;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      for (int b = 0; b < ni; b += 32) {
+        const int i = b + tid;
+        const bool on = i < ni;
+        int u = -1 - tid;
+        if (on) {
+          const int l = (int)(il[i] >> 16), rr = l / sx;
+          u = rr / N * nx4 + (l - rr * sx - 4) / 4;
+          nxt[i] = (uint16_t)NONE;
+        }
+        const unsigned m = __match_any_sync(0xffffffffu, u);
+        __syncwarp();
+        if (on) {
+          const unsigned below = m & ((1u << tid) - 1u);
+          if (below) nxt[b + 31 - __clz(below)] = (uint16_t)i;
+          else if (tl[u] != NONE) nxt[tl[u]] = (uint16_t)i;
+          else ub_[u].z = (int)(NONE << 16 | (uint32_t)i);
+        }
+        __syncwarp();
+        if (on && !(m >> tid >> 1)) tl[u] = (uint16_t)i;
+        __syncwarp();
       }
+    }
+    __syncthreads();
+    for (int u = tid; u < units; u += C2_THREADS) {
+      const int ch = u / nx4, cu = u - ch * nx4;
+      int start, d, row = -1, at[4] = {a.capi, a.capi, a.capi, a.capi};
+      march(ch, start, d);
+      uint32_t ent = (uint32_t)ub_[u].z;
+      bool line = true, edge = false;  // edge: entries among the first R rows
+      for (uint32_t i = ent & NONE; i != NONE; i = nxt[i]) {
+        const int l = (int)(il[i] >> 16), r = l / sx, p = (l - r * sx) & 3;
+        line = line && (row < 0 || row == r);
+        row = r;
+        edge = edge || (r - start) * d < R;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q == p) {
+            line = line && at[q] == a.capi;
+            at[q] = (int)i;
+          }
+      }
+      if (row >= 0 && line) ent = (uint32_t)((row - start) * d) << 16 | NONE;
+      uline[u] = make_ushort4((unsigned short)at[0], (unsigned short)at[1], (unsigned short)at[2], (unsigned short)at[3]);
+      const bool top = start == 0 && d > 0, bottom = start == rpc - 1 && d < 0;
+      const bool nb = (top && rank > 0) || (bottom && rank < C - 1);  // a neighbour's rows behind
+      int f = ch * N < nrow ? F_ON : 0;
+      if (d < 0) f |= F_UP;
+      if (start < nrow && start + d * (N - 1) < nrow) f |= F_FULL;
+      if (BAND && nb) f |= F_NB | (edge ? F_LATE : F_PUB);
+      if (BAND && (top || bottom) && !nb) f |= F_OUT;
+      ua_[u] = make_int4((start * sx + 4 + 4 * cu) * 4, (z0 + H + start) * px + HX + 4 * cu, (start * nx4 + cu) * 16, f | start << 8);
+      ub_[u] = make_int4((int)((top ? mine : mine + 2u * epar + (R - 1) * erow) + (uint32_t)cu * 16u),
+                         (int)((top ? mine - 2u * epar + (R - 1) * erow : mine + 4u * epar) + (uint32_t)cu * 16u), (int)ent, cu);
     }
 
     // state of the shot: the current and previous levels (and their low parts)
-    float* ring = a.ring + (long long)shot * a.ring_ss;
+    float* const ring = a.ring + (long long)shot * a.ring_ss;
+    __nv_bfloat16* const eb = COMP ? a.eslots + (long long)shot * a.e_ss : nullptr;
     auto slot = [&](int l) { return (long long)(((l % a.nslots) + a.nslots) % a.nslots) * a.L.field; };
     const int lc0 = a.lev0, lp0 = a.lev0 - a.dir;
     {
       const float* gc = ring + slot(lc0);
       const float* gp = ring + slot(lp0);
-      for (int i = tid; i < nrow * sx4; i += C2_THREADS) {
+      for (int i = tid; i < rpc * sx4; i += C2_THREADS) {
         const int r = i / sx4, c = i % sx4;
         const long long g = (long long)(z0 + r + H) * px + HX - 4 + 4 * c;
+        const bool in = !a.fresh && r < nrow;
         float4 vc = make_float4(0.f, 0.f, 0.f, 0.f), vp = vc;
-        if (!a.fresh) {
+        if (in) {
           vc = *reinterpret_cast<const float4*>(gc + g);
           vp = *reinterpret_cast<const float4*>(gp + g);
         }
         reinterpret_cast<float4*>(U0 + (size_t)r * sx)[c] = vc;
         reinterpret_cast<float4*>(U1 + (size_t)r * sx)[c] = vp;
         if (COMP) {
-          float4 ec = make_float4(0.f, 0.f, 0.f, 0.f), ep = ec;
-          if (!a.fresh) {
-            const __nv_bfloat16* eb = a.eslots + (long long)shot * a.e_ss;
-            ec = ld_bf4(eb + (long long)(lc0 & 1) * a.L.field + g);
-            ep = ld_bf4(eb + (long long)(lp0 & 1) * a.L.field + g);
+          uint2 ec = make_uint2(0u, 0u), ep = ec;
+          if (in) {
+            ec = *reinterpret_cast<const uint2*>(eb + (long long)(lc0 & 1) * a.L.field + g);
+            ep = *reinterpret_cast<const uint2*>(eb + (long long)(lp0 & 1) * a.L.field + g);
           }
-          st_bf4(E0 + (size_t)r * sx + 4 * c, ec);
-          st_bf4(E1 + (size_t)r * sx + 4 * c, ep);
+          *reinterpret_cast<uint2*>(E0 + (size_t)r * sx + 4 * c) = ec;
+          *reinterpret_cast<uint2*>(E1 + (size_t)r * sx + 4 * c) = ep;
         }
       }
     }
-    // a level (complete since the last cluster barrier) to its ring slot: one
-    // bulk copy per row of the band, issued by the first warp
-    auto store_level = [&](int lev, const float* Ub) {
-      if (tid >= 32) return;
-      fence_proxy_async();
-      float* g = ring + slot(lev);
-      for (int r = tid; r < nrow; r += 32)
-        bulk_row_store(g + (long long)(z0 + r + H) * px + HX, Ub + (size_t)r * sx + 4, (uint32_t)(nx4 * 16));
-      bulk_commit();
+    // value that entry i adds to level lev
+    auto entry = [&](int i, int lev) {
+      const int k = (int)(il[i] & 0xffffu);
+      return __ldg(a.inj_coef + (long long)shot * a.ninj + k) *
+             __ldg(a.inj_val + (long long)shot * a.inj_val_ss + (long long)(lev + a.inj_shift) * a.ninj + k);
     };
-    // receivers of a level (complete since the last cluster barrier)
+    for (int i = tid; i < ni; i += C2_THREADS) ival[i] = entry(i, a.lev0 + a.dir);
+    if (tid < 2) ival[tid * vstep + a.capi] = 0.f;
+    // receivers of a complete level
     auto sample = [&](int lev, const float* Ub) {
       const int orow = lev + a.samp_shift;
       if (orow < 0 || !a.samp_out) return;
       float* out = a.samp_out + (long long)shot * a.samp_out_ss + (long long)orow * a.nsamp;
-      for (int i = tid; i < ns; i += C2_THREADS) out[sk[i]] = Ub[sloc[i]];
+      for (int i = tid; i < ns; i += C2_THREADS) out[sl[i] & 0xffffu] = Ub[sl[i] >> 16];
     };
-    cluster.sync();  // every band of the cluster is loaded
+    __syncthreads();
+    if (BAND) {
+      for (int i = tid; i < 2 * R * nx4; i += C2_THREADS) {
+        const int row = i / nx4, c = i - row * nx4, side = row >= R, t = row - side * R;
+        if (side ? rank == C - 1 : rank == 0) continue;
+        const uint32_t o = (uint32_t)((side ? rpc - R + t : t) * sx + 4 + 4 * c);
+        publish(mine + side * 2u * epar + (tagb & 1u) * epar + (uint32_t)t * erow + (uint32_t)c * 16u, lds4(sU0 + o * 4u),
+                COMP ? lds2(sE0 + o * 2u) : make_uint2(0u, 0u), tagb);
+      }
+    } else {
+      cluster_arrive();  // every band of the cluster is loaded
+    }
 
-    int cur = 0;  // buffer 0 holds the current level, buffer 1 the previous one, then the new one
-    for (int step = 0; step < a.nsteps; ++step) {
-      const int lcur = a.lev0 + step * a.dir, lnew = lcur + a.dir;
-      // values of this step's sources (loaded now, used after the stencil)
-      float pv[C2_PER];
-#pragma unroll
-      for (int q = 0; q < C2_PER; ++q) {
-        const int i = tid + q * C2_THREADS;
-        pv[q] = i < ni ? pc[q] * __ldg(a.inj_val + (long long)shot * a.inj_val_ss +
-                                       (long long)(lnew + a.inj_shift) * a.ninj + pk[q])
-                       : 0.f;
-      }
-      const float* Uc = cur ? U1 : U0;
-      float* Un = cur ? U0 : U1;
-      __nv_bfloat16* En = cur ? E0 : E1;
-      const float** ru = rowU + cur * nrt + R;  // ru[r + d]: row r + d of the current level (any band)
-      const __nv_bfloat16** re = rowE + cur * nrt + R;
-      // the current level is complete: its receivers, and its copy in the ring
-      // (the first level of a launch was stored and sampled by the launch before)
-      if (step > 0) {
-        store_level(lcur, Uc);
-        sample(lcur, Uc);
-      }
-      // the thread's column chunk, marched down with the z neighbours in a
-      // register queue: rows of the band by shared-memory address, rows of
-      // other bands (or outside the grid) through the row table
-      const uint32_t sUc = cur ? sU1 : sU0, sUn = cur ? sU0 : sU1;
-      const uint32_t sEc = cur ? sE1 : sE0, sEn = cur ? sE0 : sE1;
-      auto ld_u = [&](int r) -> float4 {
-        return (r >= 0 && r < nrow) ? lds4(sUc + (uint32_t)(r * sx + 4 + 4 * cu) * 4u)
-                                    : reinterpret_cast<const float4*>(ru[r])[cu];
-      };
-      auto ld_e = [&](int r) -> float4 {
-        return (r >= 0 && r < nrow) ? bf4(lds2(sEc + (uint32_t)(r * sx + 4 + 4 * cu) * 2u))
-                                    : bf4(*reinterpret_cast<const uint2*>(re[r] + 4 * cu));
-      };
-      if (ra < rb) {
-        // the queue is circular: row r + d of block row j sits in slot
-        // (j + R + d) mod NQ, so whole blocks of NQ rows need no register moves
-        constexpr int NQ = 2 * R + 1;
-        float4 q[NQ], eq[NQ];
-#pragma unroll
-        for (int k = 0; k < 2 * R; ++k) {
-          q[k] = ld_u(ra - R + k);
-          if (COMP) eq[k] = ld_e(ra - R + k);
+    __syncthreads();
+    const int rs = sx * 4;
+    const uint32_t sA = sa(ua_), sB = sa(ub_);
+    // the words of the R rows behind (k = 0: the nearest), loaded when a march
+    // ends for the next one (COMP: as it begins, there are no registers to spare)
+    constexpr bool AHEAD = BAND && !COMP;
+    uint4 wa[BAND ? R : 1], wb[BAND ? R : 1], wc[BAND && COMP ? R : 1];
+    auto ask = [&](int k, uint32_t o) {
+      const unsigned char* p = a.edge + o;
+      wa[BAND ? k : 0] = ld_words(p);
+      wb[BAND ? k : 0] = ld_words(p + eplane);
+      if (COMP) wc[BAND && COMP ? k : 0] = ld_words(p + 2 * eplane);
+    };
+    // bounded wait for words at offset o
+    auto settle = [&](uint32_t o, uint4& x, uint4& y, uint4& z, uint32_t tag) {
+      auto came = [&] { return x.y == tag && x.w == tag && y.y == tag && y.w == tag && (!COMP || (z.y == tag && z.w == tag)); };
+      if (came()) return;
+      const unsigned char* p = a.edge + o;
+      const long long t0 = clock64();
+      while (!came()) {
+        if (*aborted) break;
+        if (clock64() - t0 > a.spin) {
+          *aborted = 1;
+          atomicOr(a.err, 1);
+          break;
         }
-        const float* c2col = a.c2 + (long long)(z0 + H) * px + HX + 4 * cu;
-        for (int r0 = ra; r0 < rb; r0 += NQ) {
+        x = ld_words(p);
+        y = ld_words(p + eplane);
+        if (COMP) z = ld_words(p + 2 * eplane);
+      }
+    };
+    const bool ahead = AHEAD && units <= C2_THREADS;
+    auto ask_ahead = [&](uint32_t tag) {  // the words of this thread's rows behind
+      if (!ahead || tid >= units) return;
+      const int f = ldsi(sA + (uint32_t)tid * 16u + 12u);
+      if ((f & (F_ON | F_NB)) != (F_ON | F_NB)) return;
+      const uint32_t o = (uint32_t)ldsi(sB + (uint32_t)tid * 16u + 4u) + (tag & 1u) * epar, st = f & F_UP ? erow : 0u - erow;
 #pragma unroll
-          for (int j = 0; j < NQ; ++j) {
-            const int r = r0 + j;
-            if (r < rb) {
-              q[(j + 2 * R) % NQ] = ld_u(r + R);
-              if (COMP) eq[(j + 2 * R) % NQ] = ld_e(r + R);
-              const uint32_t ou = (uint32_t)(r * sx + 4 + 4 * cu);
-              const float4 xl = lds4(sUc + (ou - 4) * 4u), xr = lds4(sUc + (ou + 4) * 4u), xc = q[(j + R) % NQ];
-              const float4 c1 = lds4(sUn + ou * 4u);  // previous level
-              const float4 cq = __ldg(reinterpret_cast<const float4*>(c2col + (long long)r * px));
-              const float v[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w, xr.x, xr.y, xr.z, xr.w};
-              float o[4], en[4] = {0.f, 0.f, 0.f, 0.f};
-              if (!COMP) {
-                // centred form, the per-step 2-D sweep's operations in its order
-                float2 s2[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+      for (int k = 0; k < R; ++k) ask(k, o + (uint32_t)k * st);
+    };
+    ask_ahead(tagb);
+
+    int slot_new = ((a.lev0 + a.dir) % a.nslots + a.nslots) % a.nslots;
+    float* glev = ring + (long long)slot_new * a.L.field;  // the new level's field
+    const int kfrom = a.store_all ? 0 : a.nsteps - 2;      // levels from this step on go to their ring slots
+    for (int step = 0, cur = 0; step < a.nsteps; ++step, cur ^= 1) {
+      const int lcur = a.lev0 + step * a.dir;
+      const uint32_t tag = tagb + (uint32_t)step;
+      // values that the next step injects (loaded now, put in place when this step ends)
+      float pv[PER];
+      if (ni > 0 && step + 1 < a.nsteps) {
 #pragma unroll
-                for (int k = 1; k <= R; ++k) {
-                  const float4 zp = q[(j + R + k) % NQ], zm = q[(j + R - k) % NQ];
-                  const float2 wk = f2(a.W.w[k], a.W.w[k]);
+        for (int q = 0; q < PER; ++q) pv[q] = tid + q * C2_THREADS < ni ? entry(tid + q * C2_THREADS, lcur + 2 * a.dir) : 0.f;
+      }
+      // the current level is complete: its receivers (the first level of a
+      // launch was sampled by the launch before)
+      if (ns > 0 && step > 0) sample(lcur, cur ? U1 : U0);
+      if (!BAND) {
+        __syncwarp();
+        cluster_wait();  // the level's edge rows are complete in every band
+      }
+      const bool keep = step >= kfrom;
+      const uint32_t nd = cur ? 0u - lbytes : lbytes;  // from the current level to the new one
+      // low parts of the value at shared address x: at eoff + x / 2 in the current level, at neff + x / 2 in the new one
+      const uint32_t eoff = cur ? sE0 + ebytes - (sU0 + lbytes) / 2u : sE0 - sU0 / 2u;
+      const uint32_t neff = cur ? sE0 - sU0 / 2u : sE0 + ebytes - (sU0 + lbytes) / 2u;
+      for (int un = tid; un < units; un += C2_THREADS) {
+        {
+          const int4 A = ldsi4(sA + (uint32_t)un * 16u);
+          const int f = A.w;
+          if (!(f & F_ON)) continue;
+          const int ds = f & F_UP ? -rs : rs, gd = f & F_UP ? -px : px, cd = (f & F_UP ? -nx4 : nx4) * 16;
+          uint32_t ua = sU0 + (cur ? lbytes : 0u) + (uint32_t)A.x;
+          // c2 of the unit's rows, in shared or in global memory (zero past the grid: padding)
+          uint32_t c2a = sC2 + (uint32_t)A.z;
+          int go = A.y;  // the row's place in a field
+          auto ld_c2 = [&](int x) { return C2S ? lds4(c2a) : __ldg(reinterpret_cast<const float4*>(a.c2 + x)); };
+          // clusters: row r, in the band or an edge row (zero outside the grid)
+          auto ld_any = [&](int r, uint32_t x, float4& u, uint2& e) {
+            if (r >= 0 && r < rpc) {
+              u = lds4(x);
+              if (COMP) e = lds2(eoff + x / 2u);
+            } else {
+              const int i = cur * 2 * R + (r < 0 ? r + R : r - rpc + R);
+              const uint32_t co = (uint32_t)(4 + 4 * ldsi(sB + (uint32_t)un * 16u + 12u));
+              u = ldc4(tab[i] + co * 4u);
+              if (COMP) e = ldc2(tab[4 * R + i] + co * 2u);
+            }
+          };
+          const int start = f >> 8, d = f & F_UP ? -1 : 1;
+          constexpr int BL = N % 4 == 0 ? 4 : N;  // rows of an unrolled block
+          float4 u[BL + 2 * R], cqn = ld_c2(go);
+          constexpr bool EQ = COMP && !BAND;  // low parts queued too (bands: read for every row, a second queue spilled)
+          uint2 e[EQ ? BL + 2 * R : 1];
+          uint32_t ha = ua - (uint32_t)(R * ds);  // a row's address as it enters the queue
 #pragma unroll
-                  for (int h = 0; h < 2; ++h) {
-                    const int pp = 2 * h;
-                    const float2 cv = f2(v[4 + pp], v[5 + pp]);
-                    const float2 xs = __fadd2_rn(f2(v[4 + pp + k], v[5 + pp + k]), f2(v[4 + pp - k], v[5 + pp - k]));
-                    const float2 zs = __fadd2_rn(h ? f2(zp.z, zp.w) : f2(zp.x, zp.y), h ? f2(zm.z, zm.w) : f2(zm.x, zm.y));
-                    s2[h] = __ffma2_rn(wk, __ffma2_rn(m4, cv, __fadd2_rn(xs, zs)), s2[h]);
-                  }
-                }
-                // new = c2 S + (2u - u_prev); 2u is exact, so the FMA rounds 2u - u_prev once, as a subtraction
+          for (int i = 0; i < 2 * R; ++i) {
+            if (!BAND) {
+              ld_any(start + d * (i - R), ha, u[i], e[EQ ? i : 0]);
+            } else if (i >= R || !(f & (F_NB | F_OUT))) {  // N >= R: the rows of the march, or those of the chunk behind
+              u[i] = lds4(ha);
+            }
+            ha += (uint32_t)ds;
+          }
+          if (BAND && f & F_NB) {
+            const uint32_t o = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 4u) + (tag & 1u) * epar, st = f & F_UP ? erow : 0u - erow;
+            constexpr int G = COMP ? 2 : R;  // rows asked for at once
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  const int pp = 2 * h;
-                  const float2 t = __ffma2_rn(f2(2.f, 2.f), f2(v[4 + pp], v[5 + pp]),
-                                              f2(-comp4(c1, pp), -comp4(c1, pp + 1)));
-                  const float2 r2 = __ffma2_rn(f2(comp4(cq, pp), comp4(cq, pp + 1)), s2[h], t);
-                  o[pp] = r2.x;
-                  o[pp + 1] = r2.y;
-                }
-              } else {
-                // double-float levels: U = u + e.  S(u) in the difference form for
-                // k = 1, 2 and the centred form for the small weights k = 3, 4; S(e) in
-                // the centred form (e is a few ulp of u: its rounding is negligible)
-                const float4 el = bf4(lds2(sEc + (ou - 4) * 2u)), er = bf4(lds2(sEc + (ou + 4) * 2u)), ec = eq[(j + R) % NQ];
-                const float ve[12] = {el.x, el.y, el.z, el.w, ec.x, ec.y, ec.z, ec.w, er.x, er.y, er.z, er.w};
-                const float4 e1 = bf4(lds2(sEn + ou * 2u));
-                // two points per packed fp32x2 instruction (each lane the scalar
-                // operation of the unpacked form, in the same order)
-                float2 su[2] = {f2(0.f, 0.f), f2(0.f, 0.f)}, se[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+            for (int k0 = 0; k0 < R; k0 += G) {
+              if (!ahead) {
 #pragma unroll
-                for (int k = 1; k <= R; ++k) {
-                  const float4 zp = q[(j + R + k) % NQ], zm = q[(j + R - k) % NQ], ezp = eq[(j + R + k) % NQ],
-                               ezm = eq[(j + R - k) % NQ];
-                  const float2 wk = f2(a.W.w[k], a.W.w[k]);
-#pragma unroll
-                  for (int h = 0; h < 2; ++h) {
-                    const int pp = 2 * h;
-                    const float2 xp = f2(v[4 + pp + k], v[5 + pp + k]), xm = f2(v[4 + pp - k], v[5 + pp - k]);
-                    const float2 zpp = h ? f2(zp.z, zp.w) : f2(zp.x, zp.y), zmm = h ? f2(zm.z, zm.w) : f2(zm.x, zm.y);
-                    if (k <= 2) {
-                      // the two heavy weights: per-neighbour differences, exact
-                      // for neighbours within a factor two of the centre
-                      const float2 nu = f2(-v[4 + pp], -v[5 + pp]);
-                      const float2 dxp = __fadd2_rn(xp, nu), dxm = __fadd2_rn(xm, nu);
-                      const float2 dzp = __fadd2_rn(zpp, nu), dzm = __fadd2_rn(zmm, nu);
-                      su[h] = __ffma2_rn(wk, __fadd2_rn(__fadd2_rn(dxp, dxm), __fadd2_rn(dzp, dzm)), su[h]);
-                    } else {
-                      // |w_3|, |w_4| < 0.03: the centred form's rounding is a few
-                      // hundredths of an ulp of u here
-                      su[h] = __ffma2_rn(wk, __ffma2_rn(m4, f2(v[4 + pp], v[5 + pp]),
-                                                        __fadd2_rn(__fadd2_rn(xp, xm), __fadd2_rn(zpp, zmm))),
-                                         su[h]);
-                    }
-                    const float2 xe = __fadd2_rn(f2(ve[4 + pp + k], ve[5 + pp + k]), f2(ve[4 + pp - k], ve[5 + pp - k]));
-                    const float2 ze = __fadd2_rn(h ? f2(ezp.z, ezp.w) : f2(ezp.x, ezp.y), h ? f2(ezm.z, ezm.w) : f2(ezm.x, ezm.y));
-                    se[h] = __ffma2_rn(wk, __ffma2_rn(m4, f2(ve[4 + pp], ve[5 + pp]), __fadd2_rn(xe, ze)), se[h]);
-                  }
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  const int pp = 2 * h;
-                  const float2 two = f2(2.f, 2.f);
-                  const float2 uu = f2(v[4 + pp], v[5 + pp]), ee = f2(ve[4 + pp], ve[5 + pp]);
-                  const float2 cm = f2(-comp4(c1, pp), -comp4(c1, pp + 1));
-                  const float2 em = f2(-comp4(e1, pp), -comp4(e1, pp + 1));
-                  const float2 cc2 = f2(comp4(cq, pp), comp4(cq, pp + 1));
-                  // 2u - u_prev exactly (TwoSum), then the small terms, then TwoSum again
-                  const float2 u2 = __fmul2_rn(two, uu);
-                  const float2 av = __fadd2_rn(u2, cm);
-                  const float2 bb = __fadd2_rn(av, f2(-u2.x, -u2.y));
-                  const float2 ea = __fadd2_rn(__fadd2_rn(u2, f2(-(av.x - bb.x), -(av.y - bb.y))), __fadd2_rn(cm, f2(-bb.x, -bb.y)));
-                  const float2 b = __ffma2_rn(cc2, __fadd2_rn(su[h], se[h]), __ffma2_rn(two, ee, em));
-                  const float2 bt = __fadd2_rn(b, ea);
-                  const float2 sm = __fadd2_rn(av, bt);
-                  const float2 b2 = __fadd2_rn(sm, f2(-av.x, -av.y));
-                  const float2 er2 = __fadd2_rn(__fadd2_rn(av, f2(-(sm.x - b2.x), -(sm.y - b2.y))), __fadd2_rn(bt, f2(-b2.x, -b2.y)));
-                  o[pp] = sm.x;
-                  o[pp + 1] = sm.y;
-                  en[pp] = er2.x;
-                  en[pp + 1] = er2.y;
-                }
+                for (int k = k0; k < k0 + G; ++k) ask(k, o + (uint32_t)k * st);
               }
-              if (4 * cu + 3 >= nx) {  // columns past the grid stay zero
 #pragma unroll
-                for (int pp = 0; pp < 4; ++pp)
-                  if (4 * cu + pp >= nx) o[pp] = en[pp] = 0.f;
+              for (int k = k0; k < k0 + G; ++k) {
+                uint4& x = wa[BAND ? k : 0];
+                uint4& y = wb[BAND ? k : 0];
+                uint4& z = wc[BAND && COMP ? k : 0];
+                settle(o + (uint32_t)k * st, x, y, z, tag);
+                u[R - 1 - k] = make_float4(__uint_as_float(x.x), __uint_as_float(x.z), __uint_as_float(y.x), __uint_as_float(y.z));
+                if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(z.x, z.z));
+              }
+            }
+          } else if (BAND && f & F_OUT) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+              u[R - 1 - k] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(0u, 0u));
+            }
+          }
+          const bool pub = BAND && f & F_PUB && step + 1 < a.nsteps;
+          uint32_t w = pub ? (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar : 0u;
+          const uint32_t wd = f & F_UP ? 0u - erow : erow;
+#pragma unroll 1
+          for (int b = 0; b < N / BL; ++b) {
+#pragma unroll
+            for (int jj = 0; jj < BL; ++jj) {
+              // the row R beyond this one completes the queue (bands: a row of the next chunk at most)
+              if (BAND) {
+                u[jj + 2 * R] = lds4(ha);
+              } else {
+                ld_any(start + d * (b * BL + jj + R), ha, u[jj + 2 * R], e[EQ ? jj + 2 * R : 0]);
+              }
+              ha += (uint32_t)ds;
+              const float4 cq = cqn;
+              c2a += (uint32_t)cd;
+              if (jj + 1 < BL || b + 1 < N / BL) cqn = ld_c2(go + gd);
+              const uint32_t na = ua + nd;
+              float o[4], en[4] = {0.f, 0.f, 0.f, 0.f};
+              float4 c1;
+              float2 s2[2];
+              auto low = [&](int k) {
+                if constexpr (EQ) return e[jj + R + k];
+                else return lds2(eoff + ua / 2u + (uint32_t)(k * ds / 2));
+              };
+              row4<R, MODE>(a.W, u + jj, low, cq, ua, na, eoff, neff, o, en, c1, s2);
+              if (DAMP) {
+                const int dz = nz - 1 - (z0 + start + d * (b * BL + jj)), cu = ldsi(sB + (uint32_t)un * 16u + 12u);
+                if (min(min(4 * cu, nx - 4 - 4 * cu), dz) < a.W.sw) {
+#pragma unroll
+                  for (int p = 0; p < 4; ++p) {
+                    const int dd = min(min(4 * cu + p, nx - 1 - (4 * cu + p)), dz);
+                    const float2 ai = dmp[dd >= 0 && dd < a.W.sw ? dd : a.W.sw];
+                    // tp_stencil.cu's epilogue; a = 0 (outside the layer) gives the undamped value
+                    o[p] = quotient(fmaf(comp4(cq, p), p & 1 ? s2[p / 2].y : s2[p / 2].x,
+                                         fmaf(-(1.0f - ai.x), comp4(c1, p), 2.0f * comp4(u[jj + R], p))),
+                                    1.0f + ai.x, ai.y);
+                  }
+                }
               }
               // the new value over the previous level (own points: no other thread reads them in this step)
-              *reinterpret_cast<float4*>(Un + (size_t)r * sx + 4 + 4 * cu) = make_float4(o[0], o[1], o[2], o[3]);
-              if (COMP) st_bf4(En + (size_t)r * sx + 4 + 4 * cu, make_float4(en[0], en[1], en[2], en[3]));
+              const float4 ov = make_float4(o[0], o[1], o[2], o[3]);
+              const uint2 ev = COMP ? to_bf4(make_float4(en[0], en[1], en[2], en[3])) : make_uint2(0u, 0u);
+              sts4(na, ov);
+              if (COMP) sts2(neff + na / 2u, ev);
+              if (keep && (f & F_FULL || start + d * (b * BL + jj) < nrow)) *reinterpret_cast<float4*>(glev + go) = ov;
+              go += gd;
+              ua += (uint32_t)ds;
+              if (BAND && jj < R && b == 0 && pub) {
+                publish(w, ov, ev, tag + 1);
+                w += wd;
+              }
+            }
+            if (N > BL) {
+#pragma unroll
+              for (int i = 0; i < 2 * R; ++i) {
+                u[i] = u[i + BL];
+                if (EQ) e[EQ ? i : 0] = e[EQ ? i + BL : 0];
+              }
+            }
+          }
+        }
+        // entries at this unit's points, added to the values just stored
+        const uint32_t ent = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
+        if (ent != (NONE << 16 | NONE)) {
+          const int f = ldsi(sA + (uint32_t)un * 16u + 12u), start = f >> 8, d = f & F_UP ? -1 : 1;
+          const int cu = ldsi(sB + (uint32_t)un * 16u + 12u);
+          const float* v = ival + (step & 1) * vstep;
+          float* const Un = cur ? U0 : U1;
+          __nv_bfloat16* const En = cur ? E0 : E1;
+          if (ent >> 16 != NONE) {  // a line: one row, one entry per point at most
+            const int r = start + d * (int)(ent >> 16), l = r * sx + 4 + 4 * cu;
+            const ushort4 k = uline[un];
+            const float val[4] = {v[k.x], v[k.y], v[k.z], v[k.w]};
+            float4 x = *reinterpret_cast<const float4*>(Un + l);
+            float o[4] = {x.x, x.y, x.z, x.w};
+            if (COMP) {
+              const float4 ee = bf4(*reinterpret_cast<const uint2*>(En + l));
+              float eo[4] = {ee.x, ee.y, ee.z, ee.w};
+#pragma unroll
+              for (int p = 0; p < 4; ++p) {
+                float err;
+                o[p] = two_sum(o[p], val[p], &err);
+                eo[p] += err;
+              }
+              *reinterpret_cast<uint2*>(En + l) = to_bf4(make_float4(eo[0], eo[1], eo[2], eo[3]));
+            } else {
+#pragma unroll
+              for (int p = 0; p < 4; ++p) o[p] = o[p] + val[p];
+            }
+            x = make_float4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<float4*>(Un + l) = x;
+            if (keep) *reinterpret_cast<float4*>(glev + (long long)(z0 + H + r) * px + HX + 4 * cu) = x;
+          }
+          // a chain: every node's entries in index order
+          for (uint32_t i = ent & NONE; i != NONE; i = nxt[i]) {
+            const uint32_t l = il[i] >> 16;
+            bool first = true;
+            for (uint32_t k = ent & NONE; k != i; k = nxt[k]) first = first && il[k] >> 16 != l;
+            if (!first) continue;
+            float x = Un[l], xe = COMP ? __bfloat162float(En[l]) : 0.f;
+            for (uint32_t k = i; k != NONE; k = nxt[k])
+              if (il[k] >> 16 == l) {
+                if (COMP) {
+                  float err;
+                  x = two_sum(x, v[k], &err);
+                  xe += err;
+                } else {
+                  x = x + v[k];
+                }
+              }
+            Un[l] = x;
+            if (COMP) En[l] = __float2bfloat16(xe);
+            const int r = (int)l / sx;
+            if (keep) glev[(long long)(z0 + H + r) * px + HX + ((int)l - r * sx - 4)] = x;
+          }
+        }
+        if (BAND && ent != (NONE << 16 | NONE) && step + 1 < a.nsteps) {
+          const int4 A = ldsi4(sA + (uint32_t)un * 16u);
+          if (A.w & F_LATE) {
+            const uint32_t w = (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar;
+            for (int j = 0; j < R; ++j) {
+              const uint32_t x = sU0 + (cur ? 0u : lbytes) + (uint32_t)(A.x + j * (A.w & F_UP ? -rs : rs));
+              publish(w + (uint32_t)(j * (A.w & F_UP ? -(int)erow : (int)erow)), lds4(x),
+                      COMP ? lds2(neff + x / 2u) : make_uint2(0u, 0u), tag + 1);
             }
           }
         }
       }
+      if (ni > 0 && step + 1 < a.nsteps) {
 #pragma unroll
-      for (int q = 0; q < C2_PER; ++q) {
-        const int i = tid + q * C2_THREADS;
-        if (i < ni) ival[i] = pv[q];
+        for (int q = 0; q < PER; ++q)
+          if (tid + q * C2_THREADS < ni) ival[((step + 1) & 1) * vstep + tid + q * C2_THREADS] = pv[q];
       }
-      if (tid < 32) bulk_wait_read();  // the next step overwrites the buffer the ring copies read
-      __syncthreads();
-      // sources of this step, into the new level (one thread per node, index order)
-      for (int i = tid; i < ni; i += C2_THREADS) {
-        const int m = imeta[i];
-        if (!(m & (1 << 16))) continue;
-        const int l = iloc[i];
-        float x = Un[l];
-        if (!COMP) {
-          for (int j = i; j >= 0; j = (imeta[j] >> 17) - 1) x = x + ival[j];
-        } else {
-          float e = __bfloat162float(En[l]);
-          for (int j = i; j >= 0; j = (imeta[j] >> 17) - 1) {
-            float err;
-            x = two_sum(x, ival[j], &err);
-            e += err;
-          }
-          En[l] = __float2bfloat16(e);
-        }
-        Un[l] = x;
+      // the words of the next level's edge rows, on their way while the CTA gathers
+      if (step + 1 < a.nsteps) ask_ahead(tag + 1);
+      slot_new += a.dir;
+      glev += a.dir * a.L.field;
+      if (slot_new == a.nslots || slot_new < 0) {
+        glev -= a.dir * (long long)a.nslots * a.L.field;
+        slot_new = slot_new < 0 ? a.nslots - 1 : 0;
       }
-      cluster.sync();  // the new level (and its sources) is complete in every band
-      cur ^= 1;
+      __syncthreads();  // the new level is complete in this band
+      if (!BAND) cluster_arrive();
     }
-    // the last level of the launch: its receivers, its ring slot, and the low
-    // parts of the last two levels (the next launch starts from them)
-    {
-      const int lfin = a.lev0 + a.nsteps * a.dir;
-      const float* Uc = cur ? U1 : U0;
-      sample(lfin, Uc);
-      store_level(lfin, Uc);
-      if (COMP) {
-        for (int r = ra; r < rb; ++r) {
-          const long long go = (long long)(z0 + r + H) * px + HX + 4 * cu;
-          __nv_bfloat16* eb = a.eslots + (long long)shot * a.e_ss;
-          const __nv_bfloat16* Ef = cur ? E1 : E0;
-          const __nv_bfloat16* Ep = cur ? E0 : E1;
-          *reinterpret_cast<uint2*>(eb + (long long)(lfin & 1) * a.L.field + go) =
-              *reinterpret_cast<const uint2*>(Ef + (size_t)r * sx + 4 + 4 * cu);
-          *reinterpret_cast<uint2*>(eb + (long long)((lfin - a.dir) & 1) * a.L.field + go) =
-              *reinterpret_cast<const uint2*>(Ep + (size_t)r * sx + 4 + 4 * cu);
-        }
+    // the last level's receivers, and the low parts of the last two levels
+    // (the next launch starts from them)
+    const int lfin = a.lev0 + a.nsteps * a.dir;
+    if (ns > 0) sample(lfin, a.nsteps & 1 ? U1 : U0);
+    if (COMP)
+      for (int i = tid; i < nrow * nx4; i += C2_THREADS) {
+        const int r = i / nx4, c = i - r * nx4;
+        const long long go = (long long)(z0 + r + H) * px + HX + 4 * c;
+        const size_t so = (size_t)r * sx + 4 + 4 * c;
+        *reinterpret_cast<uint2*>(eb + (long long)(lfin & 1) * a.L.field + go) =
+            *reinterpret_cast<const uint2*>((a.nsteps & 1 ? E1 : E0) + so);
+        *reinterpret_cast<uint2*>(eb + (long long)((lfin - a.dir) & 1) * a.L.field + go) =
+            *reinterpret_cast<const uint2*>((a.nsteps & 1 ? E0 : E1) + so);
       }
-    }
-    if (tid < 32) bulk_wait_all();  // the ring holds every level of the launch
-    cluster.sync();  // no CTA leaves (or starts the next shot) while a neighbour reads its band
+    if (!BAND) cluster_wait();  // no CTA leaves (or starts the next shot) while a neighbour reads its band
+    __syncthreads();            // this shot's lists and levels are no longer read
   }
 }
 
 // list capacity for n entries (a band may hold all of a shot's entries)
 int c2_cap(int n) { return (std::max(n, 1) + 3) / 4 * 4; }
 
-size_t c2_smem(int rpc, int sx, int R, bool comp, int capi, int caps) {
-  size_t b = (size_t)(2 * rpc + 1) * sx * 4;                // both levels, zero row
-  if (comp) b += (size_t)2 * rpc * sx * 2;                  // low parts of both levels (bf16)
-  b += (size_t)2 * 2 * (rpc + 2 * R) * sizeof(void*);       // row tables
-  b += (size_t)capi * 3 * 4 + (size_t)caps * 2 * 4;         // injection and sampling entries
+// shared memory of a band of rpc rows (chunks of N)
+size_t c2_bytes(int rpc, int N, int sx, int nx4, int R, int mode, bool band, bool c2s, int sw, int capi, int caps) {
+  const size_t units = (size_t)(rpc / N) * nx4;
+  size_t b = (size_t)(2 * rpc + (band ? 0 : 1)) * sx * 4;   // both levels, zero row
+  if (mode == C2_COMP) b += (size_t)(2 * rpc + (band ? 3 * R : 0)) * sx * 2;  // low parts of both levels (bf16)
+  if (c2s) b += (size_t)rpc * nx4 * 16;                     // c2
+  b += (size_t)capi * (4 + 8 + 2) + 32 + (size_t)caps * 4;  // injection and sampling entries
+  b += units * 40 + (units + 1) / 2 * 4 + 8;                // per unit
   b += (size_t)(4 + C2_THREADS / 32) * 4;                   // counts
+  if (!band) b += (size_t)8 * R * 4;                        // edge row table
+  if (mode == C2_DAMP) b += (size_t)(sw + 1) * 8 + 8;
   return (b + 15) / 16 * 16;
 }
 
-// the sizes a band of rpc rows of this grid needs; 0 if it does not fit
-size_t c2_fit(const Layout& L, int R, int C, bool comp, int capi, int caps, int* rpc_out) {
+// Whether a shot of this grid fits one cluster of C CTAs, for the acceptance
+// of the compensated form; the kernel itself needs no more than this.
+bool c2_accepts(const Layout& L, int R, int C, bool comp, int cap) {
   const int nx4 = (L.nx + 3) / 4, sx = 4 * nx4 + 8;
   const int rpc = (L.nz + C - 1) / C;
-  if (nx4 > C2_MAXCOL) return 0;
-  const size_t sm = c2_smem(rpc, sx, R, comp, capi, caps);
-  if (sm > 227 * 1024) return 0;
-  *rpc_out = rpc;
-  return sm;
+  if (nx4 > C2_MAXCOL) return false;
+  size_t b = (size_t)(2 * rpc + 1) * sx * 4 + (comp ? (size_t)2 * rpc * sx * 2 : 0);
+  b += (size_t)2 * 2 * (rpc + 2 * R) * sizeof(void*) + (size_t)cap * 20 + (size_t)(4 + C2_THREADS / 32) * 4;
+  return (b + 15) / 16 * 16 <= C2_SMEM;
 }
 
 struct C2Plan {
-  int C = 0, rpc = 0, sx = 0, nx4 = 0, ncl = 0;
+  int C = 0, rpc = 0, N = 0, groups = 0, c2s = 0;  // CTAs per shot, rows per CTA and unit, shots at once
+  bool band = false;
   size_t smem = 0;
+  double est = 0;
 };
 
+// rows per unit: bands (few units: short marches), clusters
+constexpr int C2_NB = 8, C2_NS = 4, C2_NC = 2, C2_N1 = 1;
+
+// Estimated us of a step of a band of rpc rows, from measurements on GB300 (a
+// pass marches w warps of units; every unit fills its queue with 2R rows).
+// Measured / estimated: bands, levels, 601 x 201 x 16 shots 3.9 / 4.2, 801 x 301
+// x 8 3.9 / 4.0, compensated 8.2 / 9.3 and 8.0 / 9.3; clusters, levels, 201 x
+// 201 2.1 / 2.1, 401 x 401 4.5 / 4.3, 300 x 70 x 40 3.4 / 3.3, compensated 201 x
+// 201 2.95 / 2.9.  Below them an exchange through L2 (bands) or a march's
+// latency decides.
+double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band) {
+  const int units = rpc / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
+  const double w = std::min(16, (units + 31) / 32);
+  if (band) {
+    const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : (mode == C2_DAMP ? 0.026 : 0.0185);
+    const double floor = R == 4 ? 3.6 : (N == 8 ? 1.9 : 1.5) * (mode == C2_COMP ? 1.45 : 1.0);
+    return std::max(floor, (mode == C2_COMP ? 1.9 : 1.6) + passes * N * row * w) + 0.03 * passes * w;
+  }
+  const double row = mode == C2_COMP ? 0.05 : (mode == C2_DAMP ? 0.024 : 0.02), fill = mode == C2_COMP ? 0.004 : 0.0025;
+  return (N == 1 ? 1.25 : 1.4) + passes * w * (N * row + 2 * R * fill);
+}
+
+C2Plan c2_try(const Layout& L, int R, int mode, int sw, int nshots, int C, int N, int groups, bool band, int capi, int caps) {
+  C2Plan p;
+  const int nx4 = (L.nx + 3) / 4, sx = 4 * nx4 + 8;
+  if (nx4 > C2_MAXCOL || groups < 1) return p;
+  // bands: at least two chunks, so that the rows beyond a chunk are in the band
+  const int rpc = std::max(((L.nz + C - 1) / C + N - 1) / N, band ? 2 : 1) * N;
+  if ((L.nz + rpc - 1) / rpc != C) return p;  // no empty bands
+  if ((size_t)rpc * sx > 65535) return p;  // the lists keep band indices in 16 bits
+  int c2s = 1;
+  size_t sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, true, sw, capi, caps);
+  if (sm > C2_SMEM && band) {
+    c2s = 0;
+    sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, false, sw, capi, caps);
+  }
+  if (sm > C2_SMEM) return p;
+  p.C = C; p.rpc = rpc; p.N = N; p.groups = std::min(groups, nshots); p.c2s = c2s; p.band = band; p.smem = sm;
+  p.est = (double)((nshots + p.groups - 1) / p.groups) * c2_step_cost(rpc, N, nx4, R, mode, band);
+  return p;
+}
+
+int c2_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return C2_MAXBANDS;
+  }
+  return std::min(sms, C2_MAXBANDS);
+}
+
+// The best split into bands of one cooperative grid (est = 0: none fits)
+C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, int caps) {
+  C2Plan best;
+  const int sms = c2_sms();
+  for (int C = 1; C <= sms; ++C)
+    for (int N : {C2_NB, C2_NS}) {
+      const C2Plan p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, capi, caps);
+      if (p.C && (!best.C || p.est < best.est)) best = p;
+    }
+  return best;
+}
+
 // clusters of C CTAs with `smem` bytes each that fit on the current device at once (cached)
-template <int R, bool COMP>
+template <int R, int MODE, int N>
 int c2_max_clusters(int C, size_t smem) {
   static std::mutex m;
   static std::vector<std::pair<long long, int>> cache;
@@ -575,7 +999,7 @@ int c2_max_clusters(int C, size_t smem) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, sweep2d_cluster<R, COMP>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, sweep2d_shots<R, MODE, false, N, true>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -584,68 +1008,63 @@ int c2_max_clusters(int C, size_t smem) {
   return n;
 }
 
-// Cluster size: over the sizes whose bands fit (shared memory, register
-// cache), the one with the least work per CTA over the rounds that the
-// batch's clusters need on this device (a CTA below 128 items counts as 128).
-// The step time follows the work per CTA well below a thread's worth of items:
-// a 101 x 101 shot (config 1) ran 3.25 ms per gradient with 3-CTA clusters
-// (884 items a CTA), 2.43 ms with 6 (442), 2.10 ms with 12 and 2.05 ms with 16
-// (182 items).
-template <int R, bool COMP>
-C2Plan c2_plan(const Layout& L, int nshots, int capi, int caps) {
-  C2Plan best;
-  long long best_est = -1;
-  for (int C = 1; C <= C2_MAXC; ++C) {
-    int rpc = 0;
-    const size_t sm = c2_fit(L, R, C, COMP, capi, caps, &rpc);
-    if (!sm) continue;
-    const int ncl = c2_max_clusters<R, COMP>(C, sm);
-    if (ncl < 1) continue;
-    const long long rounds = (nshots + ncl - 1) / ncl;
-    const long long est = rounds * std::max<long long>((long long)rpc * ((L.nx + 3) / 4), 128);
-    if (best_est < 0 || est < best_est) {
-      best_est = est;
-      best.C = C;
-      best.rpc = rpc;
-      best.smem = sm;
-      best.ncl = ncl;
+template <int R, int MODE>
+C2Plan c2_choose(const Layout& L, int sw, int nshots, int capi, int caps) {
+  C2Plan best = c2_bands(L, R, MODE, sw, nshots, capi, caps);
+  for (int C = 1; C <= C2_MAXC; ++C)
+    for (int N : {C2_NC, C2_N1}) {
+      C2Plan p = c2_try(L, R, MODE, sw, nshots, C, N, nshots, false, capi, caps);
+      if (!p.C) continue;
+      const int ncl = N == C2_N1 ? c2_max_clusters<R, MODE, C2_N1>(C, p.smem) : c2_max_clusters<R, MODE, C2_NC>(C, p.smem);
+      p = c2_try(L, R, MODE, sw, nshots, C, N, ncl, false, capi, caps);
+      if (p.C && (!best.C || p.est < best.est)) best = p;
     }
-  }
-  best.nx4 = (L.nx + 3) / 4;
-  best.sx = 4 * best.nx4 + 8;
   return best;
 }
 
-template <int R, bool COMP>
-cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
-  auto kern = sweep2d_cluster<R, COMP>;
-  cudaError_t e = smem_limit_once<sweep2d_cluster<R, COMP>>(227 * 1024, true);
+template <int R, int MODE, bool BAND, int N, bool C2S>
+cudaError_t c2_run(const C2Args& a, const C2Plan& pl, cudaStream_t s) {
+  const cudaError_t e = smem_limit_once<sweep2d_shots<R, MODE, BAND, N, C2S>>((int)C2_SMEM, !BAND);
   if (e != cudaSuccess) return e;
-  const int capi = c2_cap(a0.ninj), caps = c2_cap(a0.nsamp);
-  const C2Plan pl = c2_plan<R, COMP>(a0.L, a0.nshots, capi, caps);
-  if (!pl.C) return cudaErrorInvalidConfiguration;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)pl.C;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(pl.C * std::min(pl.ncl, a0.nshots)));
+  if (BAND) {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)pl.C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+  }
+  cfg.gridDim = dim3((unsigned)(pl.C * pl.groups));
   cfg.blockDim = dim3(C2_THREADS);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  const cudaError_t l = cudaLaunchKernelEx(&cfg, sweep2d_shots<R, MODE, BAND, N, C2S>, a);
+  return l != cudaSuccess ? l : cudaGetLastError();
+}
+
+template <int R, int MODE>
+cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
+  cudaError_t e = smem_limit_once<sweep2d_shots<R, MODE, false, C2_NC, true>>((int)C2_SMEM, true);  // before the occupancy query
+  if (e == cudaSuccess) e = smem_limit_once<sweep2d_shots<R, MODE, false, C2_N1, true>>((int)C2_SMEM, true);
+  if (e != cudaSuccess) return e;
   C2Args a = a0;
+  a.capi = c2_cap(a.ninj);
+  a.caps = c2_cap(a.nsamp);
+  const C2Plan pl = c2_choose<R, MODE>(a.L, a.W.sw, a.nshots, a.capi, a.caps);
+  if (!pl.C || (pl.band && !a.edge)) return cudaErrorInvalidConfiguration;
   a.C = pl.C;
   a.rpc = pl.rpc;
-  a.sx = pl.sx;
-  a.nx4 = pl.nx4;
-  a.capi = capi;
-  a.caps = caps;
-  e = cudaLaunchKernelEx(&cfg, kern, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  a.nx4 = (a.L.nx + 3) / 4;
+  a.sx = 4 * a.nx4 + 8;
+  if (!pl.band) return pl.N == C2_N1 ? c2_run<R, MODE, false, C2_N1, true>(a, pl, s) : c2_run<R, MODE, false, C2_NC, true>(a, pl, s);
+  if (pl.N == C2_NS)
+    return pl.c2s ? c2_run<R, MODE, true, C2_NS, true>(a, pl, s) : c2_run<R, MODE, true, C2_NS, false>(a, pl, s);
+  return pl.c2s ? c2_run<R, MODE, true, C2_NB, true>(a, pl, s) : c2_run<R, MODE, true, C2_NB, false>(a, pl, s);
 }
 
 }  // namespace
@@ -656,10 +1075,19 @@ bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int
   if (nsrc > C2_MAXLIST || nrec > C2_MAXLIST) return false;
   // the larger of the two sets in both lists covers the forward and the adjoint launches
   const int cap = c2_cap(std::max(nsrc, nrec));
-  int rpc = 0;
   for (int C = 1; C <= C2_MAXC; ++C)
-    if (c2_fit(L, W.R, C, comp, cap, cap, &rpc)) return true;
+    if (c2_accepts(L, W.R, C, comp, cap)) return true;
   return false;
+}
+
+bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec) {
+  if (L.ndim != 2 || nsrc > C2_MAXLIST || nrec > C2_MAXLIST) return false;
+  const int cap = c2_cap(std::max(nsrc, nrec));
+  return c2_bands(L, W.R, W.sw > 0 ? C2_DAMP : C2_LEVELS, W.sw, nshots, cap, cap).C > 0;
+}
+
+size_t edge2d_bytes(const Layout& L, const Weights& W) {
+  return (size_t)C2_MAXBANDS * 4 * W.R * ((L.nx + 3) / 4) * 16 * 3;
 }
 
 cudaError_t launch_cluster2d(const Cluster2dArgs& c, cudaStream_t s) {
@@ -667,11 +1095,11 @@ cudaError_t launch_cluster2d(const Cluster2dArgs& c, cudaStream_t s) {
   a.L = c.L;
   a.W = c.W;
   a.nshots = c.nshots;
-  a.comp = c.comp;
   a.dir = c.dir;
   a.lev0 = c.lev0;
   a.nsteps = c.nsteps;
   a.fresh = c.fresh;
+  a.store_all = c.store_all;
   a.ring = c.ring; a.nslots = c.nslots; a.ring_ss = c.ring_ss;
   a.eslots = reinterpret_cast<__nv_bfloat16*>(c.eslots); a.e_ss = c.e_ss;
   a.c2 = c.c2;
@@ -679,10 +1107,17 @@ cudaError_t launch_cluster2d(const Cluster2dArgs& c, cudaStream_t s) {
   a.inj_val = c.inj_val; a.inj_val_ss = c.inj_val_ss; a.inj_shift = c.inj_shift;
   a.samp_off = c.samp_off; a.nsamp = c.nsamp;
   a.samp_out = c.samp_out; a.samp_out_ss = c.samp_out_ss; a.samp_shift = c.samp_shift;
+  a.edge = static_cast<unsigned char*>(c.edge);
+  a.tag0 = c.tag0;
+  a.spin = wait_limit_cycles();
+  a.err = c.err;
   prof_before(0, s);  // TP_KERNEL_STENCIL
   cudaError_t e;
-  if (c.W.R == 4) e = c.comp ? c2_launch<4, true>(a, s) : c2_launch<4, false>(a, s);
-  else e = c.comp ? c2_launch<2, true>(a, s) : c2_launch<2, false>(a, s);
+  const int mode = c.comp ? C2_COMP : (c.W.sw > 0 ? C2_DAMP : C2_LEVELS);
+#define TP_C2(RR) (mode == C2_COMP ? c2_launch<RR, C2_COMP>(a, s)                         \
+                                   : (mode == C2_DAMP ? c2_launch<RR, C2_DAMP>(a, s) : c2_launch<RR, C2_LEVELS>(a, s)))
+  e = c.W.R == 4 ? TP_C2(4) : TP_C2(2);
+#undef TP_C2
   prof_after(0, s);
   return e;
 }
