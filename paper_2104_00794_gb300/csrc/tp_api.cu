@@ -151,6 +151,8 @@ struct Plan {
          o_cs = 0, o_cr = 0, o_qbar = 0, o_gacc = 0, o_sacc = 0, o_conv = 0, o_w = 0;
   // deterministic injection groups of the sources and of the receivers
   size_t o_salone = 0, o_ralone = 0, o_sshared = 0, o_rshared = 0, o_sn = 0, o_rn = 0;
+  // 3-D: the point sets by grid row (sources, receivers); the masks of both in one block
+  size_t o_pt = 0, pt_bytes = 0, o_pt_set[2] = {0, 0}, o_pt_base[2] = {0, 0}, o_pt_ent[2] = {0, 0};
   long long nf = 0;  // fields in the wavefield block
   // probed state (Q, then the forward accumulators): offsets inside the state
   // buffer, which tp_gradient_probed places at o_state of its workspace
@@ -238,6 +240,16 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
   P->o_rshared = take(cur, (size_t)ns * P->nrec * sizeof(int));
   P->o_sn = take(cur, (size_t)ns * sizeof(int));
   P->o_rn = take(cur, (size_t)ns * sizeof(int));
+  if (P->L.ndim == 3) {
+    const size_t segs = (size_t)ns * pt_segs(P->L), words = (size_t)ns * pt_tiles(P->L) * pt_words(P->L);
+    P->o_pt = cur;
+    for (int i = 0; i < 2; ++i) P->o_pt_set[i] = take(cur, segs * 16 + words * 4 + (size_t)ns * 8);
+    P->pt_bytes = cur - P->o_pt;
+    for (int i = 0; i < 2; ++i) {
+      P->o_pt_base[i] = take(cur, segs * sizeof(int));
+      P->o_pt_ent[i] = take(cur, (size_t)ns * (i ? P->nrec : P->nsrc) * sizeof(int));
+    }
+  }
   P->c2_bytes = fb + (P->L.ndim == 2 ? (size_t)8 * P->L.plane * sizeof(float) : 0);  // + rows that a 2-D band's last chunk reads
   P->o_c2 = take(cur, P->c2_bytes);
   P->form = g->form;
@@ -338,6 +350,21 @@ tp_status check_ws(const Plan& P, void* ws, size_t ws_bytes) {
   return TP_OK;
 }
 
+// the source (0) or receiver (1) set of a 3-D plan by grid row
+PointTiles point_tiles(const Ctx& c, int set) {
+  const Plan& P = c.P;
+  const size_t segs = (size_t)P.nshots * pt_segs(P.L), words = (size_t)P.nshots * pt_tiles(P.L) * pt_words(P.L);
+  char* b = c.at<char>(P.o_pt_set[set]);
+  PointTiles t;
+  t.mask = reinterpret_cast<unsigned long long*>(b);
+  t.dup = t.mask + segs;
+  t.tile = reinterpret_cast<unsigned int*>(b + segs * 16);
+  t.count = reinterpret_cast<int*>(b + segs * 16 + words * 4);
+  t.base = c.at<int>(P.o_pt_base[set]);
+  t.ent = c.at<int>(P.o_pt_ent[set]);
+  return t;
+}
+
 // Common set-up: coefficient field, point offsets, CFL check.
 tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float* vel) {
   const Plan& P = c.P;
@@ -351,13 +378,21 @@ tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float*
                          c.at<float>(P.o_cs), c.err(), c.st));
   TRY(launch_prep_points(P.L, P.W, geo->rec, (long long)P.nshots * P.nrec, vel, dt2, c.at<long long>(P.o_roff),
                          c.at<float>(P.o_cr), c.err(), c.st));
-  // injection groups; the wavefield block (at least one field per shot, zeroed
-  // by every operation after the set-up) serves as the count scratch
-  int* cnt = c.at<int>(P.o_f);
-  TRY(launch_point_groups(c.at<long long>(P.o_soff), P.nsrc, P.nshots, P.L.field, cnt, c.at<unsigned char>(P.o_salone),
-                          c.at<int>(P.o_sshared), c.at<int>(P.o_sn), c.st));
-  TRY(launch_point_groups(c.at<long long>(P.o_roff), P.nrec, P.nshots, P.L.field, cnt, c.at<unsigned char>(P.o_ralone),
-                          c.at<int>(P.o_rshared), c.at<int>(P.o_rn), c.st));
+  if (P.L.ndim == 3) {  // the sweeps inject
+    TRY(cudaMemsetAsync(c.at<char>(P.o_pt), 0, P.pt_bytes, c.st));
+    TRY(launch_point_tiles(P.L, c.at<long long>(P.o_soff), P.nsrc, P.nshots, point_tiles(c, 0),
+                           c.at<unsigned char>(P.o_salone), c.at<int>(P.o_sshared), c.at<int>(P.o_sn), c.st));
+    TRY(launch_point_tiles(P.L, c.at<long long>(P.o_roff), P.nrec, P.nshots, point_tiles(c, 1),
+                           c.at<unsigned char>(P.o_ralone), c.at<int>(P.o_rshared), c.at<int>(P.o_rn), c.st));
+  } else {
+    // injection groups; the wavefield block (at least one field per shot, zeroed
+    // by every operation after the set-up) serves as the count scratch
+    int* cnt = c.at<int>(P.o_f);
+    TRY(launch_point_groups(c.at<long long>(P.o_soff), P.nsrc, P.nshots, P.L.field, cnt,
+                            c.at<unsigned char>(P.o_salone), c.at<int>(P.o_sshared), c.at<int>(P.o_sn), c.st));
+    TRY(launch_point_groups(c.at<long long>(P.o_roff), P.nrec, P.nshots, P.L.field, cnt,
+                            c.at<unsigned char>(P.o_ralone), c.at<int>(P.o_rshared), c.at<int>(P.o_rn), c.st));
+  }
   float vmax = g->vmax;
   if (!(vmax > 0.f)) {
     TRY(launch_vmax(vel, (long long)g->nx * g->ny * g->nz, &c.scal()->vmax_bits, c.st));
@@ -377,24 +412,27 @@ tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float*
 // the increment fields (TP_FORM_INCREMENT), one per shot
 Fam inc_fam(const Plan& P) { return Fam{P.o_w, P.nshots, 1}; }
 
-tp_status step(const Ctx& c, const Fam& f, int cur, int old, int out) {
+// one step; in 3-D with its sampling and injection (pt)
+tp_status step(const Ctx& c, const Fam& f, int cur, int old, int out, const PointArgs& pt) {
   const FieldRef c2 = c.ref(Fam{c.P.o_c2, 1, 0}, 0);
   if (c.P.form == TP_FORM_INCREMENT) {
     const Fam fw = inc_fam(c.P);
     StencilArgs a{c.ref(f, cur), c.ref(fw, 0), c2, c.ptr(f, out), c.ss(f), c.P.nshots, c.ptr(fw, 0), c.ss(fw)};
+    a.pt = pt;
     TRY(launch_stencil(MODE_INC, c.P.L, c.P.W, a, c.st, c.err()));
   } else {
     StencilArgs a{c.ref(f, cur), c.ref(f, old), c2, c.ptr(f, out), c.ss(f), c.P.nshots};
+    a.pt = pt;
     TRY(launch_stencil(MODE_STEP, c.P.L, c.P.W, a, c.st, c.err()));
   }
   return TP_OK;
 }
 
 // sampling of `samp` at offsets soff into out (may be null), injection into `inj`
-tp_status point(const Ctx& c, const float* samp, long long samp_ss, const long long* soff, int nsamp, float* out,
-                long long out_ss, float* inj, long long inj_ss, const long long* ioff, const float* icoef, int ninj,
-                const float* ival, long long ival_ss, double* acc = nullptr, const float* aval = nullptr,
-                long long aval_ss = 0) {
+PointArgs point_args(const Ctx& c, const float* samp, long long samp_ss, const long long* soff, int nsamp, float* out,
+                     long long out_ss, float* inj, long long inj_ss, const long long* ioff, const float* icoef, int ninj,
+                     const float* ival, long long ival_ss, double* acc = nullptr, const float* aval = nullptr,
+                     long long aval_ss = 0) {
   PointArgs a{};
   a.nshots = c.P.nshots;
   a.field_samp = samp; a.samp_ss = samp_ss; a.samp_off = soff; a.nsamp = samp ? nsamp : 0;
@@ -405,6 +443,7 @@ tp_status point(const Ctx& c, const float* samp, long long samp_ss, const long l
     a.inj_alone = c.at<unsigned char>(src ? c.P.o_salone : c.P.o_ralone);
     a.inj_shared = c.at<int>(src ? c.P.o_sshared : c.P.o_rshared);
     a.inj_nshared = c.at<int>(src ? c.P.o_sn : c.P.o_rn);
+    if (c.P.L.ndim == 3) a.tiles = point_tiles(c, src ? 0 : 1);
   }
   if (inj && c.P.form == TP_FORM_INCREMENT) {  // sources enter the increment as well as the new level
     a.field_inj2 = c.ptr(inc_fam(c.P), 0);
@@ -412,8 +451,7 @@ tp_status point(const Ctx& c, const float* samp, long long samp_ss, const long l
   }
   a.inj_val = ival; a.inj_val_ss = ival_ss;
   a.acc = acc; a.acc_val = aval; a.acc_val_ss = aval_ss;
-  TRY(launch_point(a, c.st));
-  return TP_OK;
+  return a;
 }
 
 #define TRYS(expr)                    \
@@ -482,15 +520,18 @@ tp_status forward_loop(const Ctx& c, const Fam& f, LevelFn level, const float* w
   if (P.form == TP_FORM_INCREMENT)  // u[1] - u[0] = 0
     TRY(cudaMemsetAsync(c.at<char>(P.o_w), 0, (size_t)P.nshots * P.L.field * sizeof(float), c.st));
   for (int t = 1; t <= P.nt - 2; ++t) {
-    TRYS(step(c, f, level(t), level(t - 1), level(t + 1)));
-    TRYS(point(c, d ? c.ptr(f, level(t)) : nullptr, ss, c.at<long long>(P.o_roff), P.nrec,
-               d ? d + (long long)t * P.nrec : nullptr, dss, c.ptr(f, level(t + 1)), ss, c.at<long long>(P.o_soff),
-               c.at<float>(P.o_cs), P.nsrc, wav + (long long)t * P.nsrc, wss));
+    const PointArgs pt =
+        point_args(c, d ? c.ptr(f, level(t)) : nullptr, ss, c.at<long long>(P.o_roff), P.nrec,
+                   d ? d + (long long)t * P.nrec : nullptr, dss, c.ptr(f, level(t + 1)), ss, c.at<long long>(P.o_soff),
+                   c.at<float>(P.o_cs), P.nsrc, wav + (long long)t * P.nsrc, wss);
+    TRYS(step(c, f, level(t), level(t - 1), level(t + 1), pt));
+    if (P.L.ndim == 2) TRY(launch_point(pt, c.st));
     TRYS(after_level(t + 1));
   }
   if (d)
-    TRYS(point(c, c.ptr(f, level(P.nt - 1)), ss, c.at<long long>(P.o_roff), P.nrec, d + (long long)(P.nt - 1) * P.nrec,
-               dss, nullptr, 0, nullptr, nullptr, 0, nullptr, 0));
+    TRY(launch_point(point_args(c, c.ptr(f, level(P.nt - 1)), ss, c.at<long long>(P.o_roff), P.nrec,
+                                d + (long long)(P.nt - 1) * P.nrec, dss, nullptr, 0, nullptr, nullptr, 0, nullptr, 0),
+                     c.st));
   return TP_OK;
 }
 
@@ -525,19 +566,23 @@ tp_status adjoint_loop(const Ctx& c, const Fam& f, LevelFn level, const float* s
   if (P.form == TP_FORM_INCREMENT)  // lambda[nt] - lambda[nt+1] = 0
     TRY(cudaMemsetAsync(c.at<char>(P.o_w), 0, (size_t)P.nshots * P.L.field * sizeof(float), c.st));
   for (int j = P.nt - 1; j >= 2; --j) {
+    const PointArgs pt =
+        point_args(c, samp ? c.ptr(f, level(j + 1)) : nullptr, ss, c.at<long long>(P.o_soff), P.nsrc,
+                   q_out ? q_out + (long long)j * P.nsrc : nullptr, qss, c.ptr(f, level(j)), ss, c.at<long long>(P.o_roff),
+                   c.at<float>(P.o_cr), P.nrec, s + (long long)j * P.nrec, sss, acc,
+                   aval ? aval + (long long)j * P.nsrc : nullptr, qss);
     if constexpr (std::is_same_v<StepFn, std::nullptr_t>)
-      TRYS(step(c, f, level(j + 1), level(j + 2), level(j)));
+      TRYS(step(c, f, level(j + 1), level(j + 2), level(j), pt));
     else
-      TRYS(step_j(j));
-    TRYS(point(c, samp ? c.ptr(f, level(j + 1)) : nullptr, ss, c.at<long long>(P.o_soff), P.nsrc,
-               q_out ? q_out + (long long)j * P.nsrc : nullptr, qss, c.ptr(f, level(j)), ss, c.at<long long>(P.o_roff),
-               c.at<float>(P.o_cr), P.nrec, s + (long long)j * P.nrec, sss, acc,
-               aval ? aval + (long long)j * P.nsrc : nullptr, qss));
+      TRYS(step_j(j, pt));
+    if (P.L.ndim == 2) TRY(launch_point(pt, c.st));
     TRYS(after_level(j));
   }
   if (samp)
-    TRYS(point(c, c.ptr(f, level(2)), ss, c.at<long long>(P.o_soff), P.nsrc, q_out ? q_out + P.nsrc : nullptr, qss,
-               nullptr, 0, nullptr, nullptr, 0, nullptr, 0, acc, aval ? aval + P.nsrc : nullptr, qss));
+    TRY(launch_point(point_args(c, c.ptr(f, level(2)), ss, c.at<long long>(P.o_soff), P.nsrc,
+                                q_out ? q_out + P.nsrc : nullptr, qss, nullptr, 0, nullptr, nullptr, 0, nullptr, 0, acc,
+                                aval ? aval + P.nsrc : nullptr, qss),
+                     c.st));
   return TP_OK;
 }
 
@@ -948,12 +993,13 @@ tp_status tp_gradient_full(const tp_grid* grid, const tp_geom* geom, const float
     // the same arithmetic as the separate sweep (lambda[nt] = 0 and u[1] = 0
     // make the first and the omitted last term exactly zero)
     const FieldRef c2 = c.ref(Fam{P.o_c2, 1, 0}, 0);
-    auto fused = [&](int j) -> tp_status {
+    auto fused = [&](int j, const PointArgs& pt) -> tp_status {
       StencilArgs a{c.ref(fl, lam(j + 1)), c.ref(fl, lam(j + 2)), c2, c.ptr(fl, lam(j)), c.ss(fl), P.nshots};
       a.img = c.ref(fh, j);
       a.gin = c.ref(fG, 0);
       a.gout = c.ptr(fG, 0);
       a.gout_ss = c.ss(fG);
+      a.pt = pt;
       TRY(launch_stencil(MODE_STEP_IMG, P.L, P.W, a, c.st, c.err()));
       return TP_OK;
     };

@@ -89,6 +89,45 @@ struct FieldRef {
   }
 };
 
+// 3-D: the entries of a point set by grid row, for the sweep that injects them
+// into the points it forms.  A segment is 64 consecutive nodes of a row
+// (segment (z * ny + y) * ntx + x / 64 of a shot, ntx = ceil(nx / 64)); entry e
+// of segment s (in node order) is ent[shot][base[s] + e]: the index of the only
+// entry at that node, or -1 where several share it (they are in `shared`).
+// tile: a bit per plane for every 64 x 16 column of the grid.
+constexpr int PT_X = 64, PT_Y = 16;
+struct PointTiles {
+  unsigned int* tile;         // [shot][ceil(ny / 16) * ntx][ceil(nz / 32)]
+  unsigned long long* mask;   // [shot][segments]: nodes with entries
+  unsigned long long* dup;    // [shot][segments]: nodes with several
+  int* base;                  // [shot][segments]
+  int* ent;                   // [shot][entries]
+  int* count;                 // [shot][2] scratch: entries placed, entries that share a node
+};
+__host__ __device__ inline int pt_tx(const Layout& L) { return (L.nx + PT_X - 1) / PT_X; }
+__host__ __device__ inline int pt_words(const Layout& L) { return (L.nz + 31) / 32; }
+inline long long pt_tiles(const Layout& L) { return (long long)pt_tx(L) * ((L.ny + PT_Y - 1) / PT_Y); }
+inline long long pt_segs(const Layout& L) { return (long long)L.nz * L.ny * pt_tx(L); }
+
+// One thread per point of two independent sets, all shots:
+//   sample: samp_out[s][t_s][j] = field_samp[s][samp_off[s][j]]           (j < nsamp)
+//   inject: field_inj[s][inj_off[s][k]] += inj_coef[s][k] * inj_val[s][t_i][k]  (k < ninj)
+//   srcacc (optional): acc[s][j] += sampled value * acc_val[s][t_a][j]
+// Injection is deterministic: entries alone at their node (inj_alone[s][k])
+// are added by their own thread, the others (inj_shared[s][0 .. inj_nshared[s]),
+// in index order) by one thread per shot, one after the other.
+struct PointArgs {
+  int nshots;
+  const float* field_samp; long long samp_ss;
+  const long long* samp_off; int nsamp; float* samp_out; long long samp_out_ss;  // already offset to t
+  float* field_inj; long long inj_ss;
+  float* field_inj2; long long inj2_ss;  // optional second target (the increment field)
+  const long long* inj_off; const float* inj_coef; int ninj;
+  const float* inj_val; long long inj_val_ss;  // already offset to t
+  const unsigned char* inj_alone; const int* inj_shared; const int* inj_nshared;
+  double* acc; const float* acc_val; long long acc_val_ss;  // may be null
+  PointTiles tiles;  // 3-D: where the injection entries are
+};
 // MODE_STEP : out = 2 src - p1 + p2 * S(src)          (leapfrog, p1 = older level, p2 = c2)
 // MODE_INC  : w' = p1 + p2 * S(src), out = src + w', and w' is stored to out2
 //             (the increment form: p1 = out2 = the increment u[t] - u[t-1])
@@ -109,6 +148,7 @@ struct StencilArgs {
   FieldRef gin{};            // MODE_STEP_IMG: the accumulator read
   float* gout = nullptr;     // MODE_STEP_IMG: the accumulator written (shot 0), per-shot stride gout_ss
   long long gout_ss = 0;
+  PointArgs pt{};            // 3-D steps: sampling of src and injection into out (and out2), in the same launch
 };
 cudaError_t launch_stencil(int mode, const Layout& L, const Weights& W, const StencilArgs& a,
                            cudaStream_t s, int* err);
@@ -188,29 +228,14 @@ cudaError_t launch_vmax(const float* vel, long long n, unsigned int* out_bits, c
 cudaError_t launch_prep_points(const Layout& L, const Weights& W, const int64_t* idx, long long n, const float* vel,
                                double dt2, long long* off, float* cinj, int* err, cudaStream_t s);
 
-// One thread per point of two independent sets, all shots:
-//   sample: samp_out[s][t_s][j] = field_samp[s][samp_off[s][j]]           (j < nsamp)
-//   inject: field_inj[s][inj_off[s][k]] += inj_coef[s][k] * inj_val[s][t_i][k]  (k < ninj)
-//   srcacc (optional): acc[s][j] += sampled value * acc_val[s][t_a][j]
-// Injection is deterministic: entries alone at their node (inj_alone[s][k])
-// are added by their own thread, the others (inj_shared[s][0 .. inj_nshared[s]),
-// in index order) by one thread per shot, one after the other.
-struct PointArgs {
-  int nshots;
-  const float* field_samp; long long samp_ss;
-  const long long* samp_off; int nsamp; float* samp_out; long long samp_out_ss;  // already offset to t
-  float* field_inj; long long inj_ss;
-  float* field_inj2; long long inj2_ss;  // optional second target (the increment field)
-  const long long* inj_off; const float* inj_coef; int ninj;
-  const float* inj_val; long long inj_val_ss;  // already offset to t
-  const unsigned char* inj_alone; const int* inj_shared; const int* inj_nshared;
-  double* acc; const float* acc_val; long long acc_val_ss;  // may be null
-};
 cudaError_t launch_point(const PointArgs& a, cudaStream_t s);
 // alone / shared / nshared of a point set (per_shot entries per shot) from the
 // padded offsets; cnt_scratch: nshots * field ints of scratch
 cudaError_t launch_point_groups(const long long* off, int per_shot, int nshots, long long field, int* cnt_scratch,
                                 unsigned char* alone, int* shared, int* nshared, cudaStream_t s);
+// 3-D: the same set as `tiles` (tile, mask, dup and count zero on entry), shared and nshared; flags: n bytes of scratch
+cudaError_t launch_point_tiles(const Layout& L, const long long* off, int per_shot, int nshots, const PointTiles& tiles,
+                               unsigned char* flags, int* shared, int* nshared, cudaStream_t s);
 
 cudaError_t launch_probes(int kind, int nt, int r, uint64_t seed, int shot0, int nshots,
                           const float* Z_user, float* Q, cudaStream_t s);

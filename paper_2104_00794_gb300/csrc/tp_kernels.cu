@@ -134,6 +134,77 @@ __global__ void __launch_bounds__(256) point_group_kernel(const long long* __res
   if (tid == 0) nshared[s] = base_cnt;
 }
 
+// 3-D point sets by grid row (PointTiles).  Before, a field of counts per set
+// (67 MB to clear at 256^3) and one CTA per shot over all entries (156 us for
+// 65536 receivers) prepared a separate injection launch for every step.
+struct PtPos {
+  long long seg;
+  int bit;
+};
+__device__ __forceinline__ PtPos pt_pos(const Layout& L, long long o, int* tile_word, int* tile_bit) {
+  const long long z = o / L.plane - H, rem = o % L.plane;
+  const int y = (int)(rem / L.px) - H, x = (int)(rem % L.px) - HX;
+  const int ntx = pt_tx(L);
+  if (tile_word) {
+    *tile_word = ((y / PT_Y) * ntx + x / PT_X) * pt_words(L) + (int)(z / 32);
+    *tile_bit = (int)(z % 32);
+  }
+  return PtPos{(z * L.ny + y) * ntx + x / PT_X, x % PT_X};
+}
+
+// step 0: masks, and flags[k] = 1 for the first entry of a segment; step 1:
+// these place their segment; step 2: every entry writes its slot
+__global__ void point_tiles_kernel(Layout L, const long long* __restrict__ off, long long n, int per_shot,
+                                   long long segs, long long tile_words, PointTiles t, unsigned char* flags, int step) {
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+    const long long o = off[k], s = k / per_shot;
+    if (o < 0) {
+      flags[k] = 0;
+      continue;
+    }
+    int tw = 0, tb = 0;
+    const PtPos p = pt_pos(L, o, &tw, &tb);
+    const long long seg = s * segs + p.seg;
+    const unsigned long long bit = 1ULL << p.bit;
+    if (step == 0) {
+      const unsigned long long had = atomicOr(t.mask + seg, bit);
+      if (had & bit) atomicOr(t.dup + seg, bit);
+      flags[k] = had == 0 ? 1 : 0;
+      atomicOr(t.tile + s * tile_words + tw, 1u << tb);
+    } else if (step == 1) {
+      if (flags[k]) t.base[seg] = atomicAdd(t.count + 2 * s, __popcll(t.mask[seg]));
+    } else {
+      const bool several = (t.dup[seg] & bit) != 0;
+      t.ent[s * per_shot + t.base[seg] + __popcll(t.mask[seg] & (bit - 1))] = several ? -1 : (int)(k % per_shot);
+      flags[k] = several ? 2 : 0;
+      if (several) atomicAdd(t.count + 2 * s + 1, 1);
+    }
+  }
+}
+
+// one block per shot: the entries that share a node (flags[k] = 2), in index order
+__global__ void __launch_bounds__(256) point_shared_kernel(const unsigned char* __restrict__ flags, int per_shot,
+                                                           const int* __restrict__ count, int* shared, int* nshared) {
+  __shared__ int warp_cnt[8];
+  const int s = blockIdx.x, tid = threadIdx.x;
+  int base = 0;
+  if (count[2 * s + 1] > 0)
+    for (int b = 0; b < per_shot; b += 256) {
+      const bool dup = b + tid < per_shot && flags[(long long)s * per_shot + b + tid] == 2;
+      const unsigned m = __ballot_sync(0xffffffffu, dup);
+      if ((tid & 31) == 0) warp_cnt[tid >> 5] = __popc(m);
+      __syncthreads();
+      int before = base;
+      for (int w = 0; w < 8; ++w) {
+        if (w < (tid >> 5)) before += warp_cnt[w];
+        base += warp_cnt[w];
+      }
+      if (dup) shared[(long long)s * per_shot + before + __popc(m & ((1u << (tid & 31)) - 1u))] = b + tid;
+      __syncthreads();
+    }
+  if (tid == 0) nshared[s] = base;
+}
+
 // SplitMix64 (Steele, Lea & Flood 2014): the n-th output of a generator whose
 // state starts at s is mix(s + n * 0x9E3779B97F4A7C15).
 __device__ __forceinline__ uint64_t sm64(uint64_t s, uint64_t n) {
@@ -363,6 +434,17 @@ cudaError_t launch_point_groups(const long long* off, int per_shot, int nshots, 
   }
   prof_after(5, s);
   return e;
+}
+
+cudaError_t launch_point_tiles(const Layout& L, const long long* off, int per_shot, int nshots, const PointTiles& t,
+                               unsigned char* flags, int* shared, int* nshared, cudaStream_t s) {
+  prof_before(5, s);
+  const long long n = (long long)nshots * per_shot, tile_words = pt_tiles(L) * pt_words(L);
+  for (int step = 0; step < 3; ++step)
+    point_tiles_kernel<<<grid_for(n, 256), 256, 0, s>>>(L, off, n, per_shot, pt_segs(L), tile_words, t, flags, step);
+  point_shared_kernel<<<nshots, 256, 0, s>>>(flags, per_shot, t.count, shared, nshared);
+  prof_after(5, s);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_point(const PointArgs& a, cudaStream_t s) {

@@ -5,7 +5,7 @@
 // the sum over the six neighbours at distance k of (neighbour - u).  The
 // kernel is HBM-bound (16 B per point: read u, u_old, c2; write out).  Design:
 //   * work items = (64 x 16 x-y tile, shot, z chunk); each tile column is cut
-//     into as many equal z chunks as keep one wave of 2 CTAs per SM busy, and
+//     into equal z chunks (launch_c says how many), and
 //     items are ordered chunk-major, so neighbouring tiles are swept at the
 //     same depths at the same time and their shared halo planes hit in L2
 //     (a balanced linear split over (tile, z) left neighbours at different
@@ -15,14 +15,26 @@
 //     [16+2R][64+8] and the u_old / c2 planes [16][64] into a ring of shared
 //     memory stages guarded by mbarriers (full: TMA transaction bytes,
 //     empty: one arrival per consumer warp), R+1+3 u planes deep so three
-//     planes are in flight while R+1 are resident;
+//     planes are in flight while R+1 are resident.  One pair of barriers serves
+//     a plane's u, u_old and c2 copies: a thread's wait and expect take 140 ns,
+//     each further copy 32 ns (measured), and with a pair for u and one for
+//     u_old / c2 the producer paced the sweep (0.37 us a plane);
 //   * 256 consumer threads own 4 consecutive x points each; the z neighbours
 //     live in a register queue of 2R+1 float4, x/y neighbours are read from
 //     the resident centre plane (x halo from the box, zero halo layers from
 //     the padded layout), so every value crosses HBM about once per step;
+//   * sources and receivers are handled in the same launch: all consumer threads
+//     sample the source field while the first planes are on their way, and a
+//     thread injects into its own points after its item (PointTiles).  Launches
+//     are programmatic: a sweep's CTAs start up as the previous one's leave.
+//     us per step (forward, order 8 / ragged: order 4), separate point launches
+//     and barrier pairs -> this: 64^3 18.8 -> 6.9, 128^3 19.7 -> 9.9,
+//     131 x 119 x 107 x 2 23.3 -> 14.6, 192 x 160 x 144 23.8 -> 15.8,
+//     256^3 62 -> 50 (HBM: 39.5 us for 16 B per point at the copy rate);
+//     two rows per thread (a third less shared-memory reading) 10 % slower;
 //   * the full-storage adjoint (MODE_STEP_IMG) also stages the history level
-//     u[j] (haloed, on the u stages' barriers) and the gradient accumulator (on
-//     the u_old / c2 stages'), keeps u[j]'s z neighbours in a second register
+//     u[j] (haloed, on the u stages) and the gradient accumulator (on
+//     the u_old / c2 stages), keeps u[j]'s z neighbours in a second register
 //     queue, and adds the imaging term of Eq. 3, lambda[j+1] * S(u[j]), in the
 //     same pass: 28 B per point instead of 16 + 16 in two sweeps, one CTA per SM;
 //   * every wait is bounded (clock64); on a timeout the CTA sets bit 0 of
@@ -47,7 +59,7 @@ constexpr int IMG_LA = 5;
 
 // Tile BX x BY (BX/4 * BY == NCONS) and LA planes of lookahead.  IMG: the
 // fused step-and-imaging sweep, with a second haloed field (its planes share
-// the u stages' barriers) and the accumulator (sharing the u_old / c2 stages').
+// the u stages) and the accumulator (sharing the u_old / c2 stages).
 template <int R, int BX_, int BY_, int LA_, bool IMG_ = false>
 struct Cfg {
   static constexpr int BX = BX_, BY = BY_, LA = LA_;
@@ -62,7 +74,7 @@ struct Cfg {
   static constexpr int UFL = UW * UH, PFL = BX * BY;
   static constexpr uint32_t UBYTES = UFL * 4, PBYTES = PFL * 4;
   static constexpr size_t BAR_OFF = (size_t)(NFU * NSU * UFL + NFP * NSP * PFL) * 4;
-  static constexpr size_t SMEM = BAR_OFF + (size_t)(2 * NSU + 2 * NSP) * 8 + 16;
+  static constexpr size_t SMEM = BAR_OFF + (size_t)(2 * NSU) * 8 + 16;
 };
 
 struct TmaArgs {
@@ -79,6 +91,7 @@ struct TmaArgs {
   int nshots, ntx, nty;
   int nzc, zchunk;  // each tile column is cut into nzc chunks of zchunk planes
   long long items;  // tiles x shots x nzc work items
+  PointArgs pt;     // sampling of the source field, injection into out (and out2)
   long long spin;   // limit of the role waits (cycles); the drain waits use DEFAULT_WAIT_CYCLES
   int* err;
 };
@@ -94,6 +107,7 @@ __device__ __forceinline__ void bar_expect_tx(uint32_t b, uint32_t bytes) {
 __device__ __forceinline__ void bar_arrive(uint32_t b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
 }
+// a poll of a phase; the thread may sleep in hardware between polls
 __device__ __forceinline__ bool bar_try(uint32_t b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -103,8 +117,7 @@ __device__ __forceinline__ bool bar_try(uint32_t b, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// non-blocking probe of a phase (mbarrier.try_wait may suspend the thread in
-// hardware until the phase completes, longer than a short wait limit)
+// the same without sleeping
 __device__ __forceinline__ bool bar_test(uint32_t b, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -114,17 +127,17 @@ __device__ __forceinline__ bool bar_test(uint32_t b, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// bounded wait; false on timeout or when another role has aborted.  With the
-// default limit it polls with try_wait (the thread sleeps in hardware between
-// polls); with a shorter one, set through tp_set_wait_limit, with test_wait,
-// so that the limit is what ends the wait.
+// bounded wait; false on timeout or when another role has aborted.  A limit
+// shorter than the default, set through tp_set_wait_limit, polls without
+// sleeping, so that the limit is what ends the wait.
 __device__ __forceinline__ bool bar_wait(uint32_t b, uint32_t parity, volatile int* abort_flag, long long limit) {
   const bool quick = limit < DEFAULT_WAIT_CYCLES;
-  if (quick ? bar_test(b, parity) : bar_try(b, parity)) return true;
-  const long long t0 = clock64();
+  long long t0 = 0;
   while (!(quick ? bar_test(b, parity) : bar_try(b, parity))) {
     if (*abort_flag) return false;
-    if (clock64() - t0 > limit) {
+    const long long t = clock64();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > limit) {
       *abort_flag = 1;
       return false;
     }
@@ -186,11 +199,9 @@ __device__ __forceinline__ Seg segment(const TmaArgs& a, long long item) {
 // IEEE round-to-nearest operation of the scalar form, in the same order.
 template <int R, int RW>
 __device__ __forceinline__ void star4(const float4* Uc, const float4 (&q)[2 * R + 1], int cidx, const Weights& W,
-                                      float (&v)[12], float (&s4)[4]) {
-  const float4 xl = Uc[cidx - 1], xc = Uc[cidx], xr = Uc[cidx + 1];
-  v[0] = xl.x; v[1] = xl.y; v[2] = xl.z; v[3] = xl.w;
-  v[4] = xc.x; v[5] = xc.y; v[6] = xc.z; v[7] = xc.w;
-  v[8] = xr.x; v[9] = xr.y; v[10] = xr.z; v[11] = xr.w;
+                                      float (&s4)[4]) {
+  const float4 xl = Uc[cidx - 1], xc = q[R], xr = Uc[cidx + 1];
+  const float v[12] = {xl.x, xl.y, xl.z, xl.w, xc.x, xc.y, xc.z, xc.w, xr.x, xr.y, xr.z, xr.w};
   float2 s2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   const float2 m6 = make_float2(-6.f, -6.f);
 #pragma unroll
@@ -202,7 +213,9 @@ __device__ __forceinline__ void star4(const float4* Uc, const float4 (&q)[2 * R 
     for (int h = 0; h < 2; ++h) {
       const int p = 2 * h;
       const float2 c = make_float2(v[4 + p], v[5 + p]);
-      const float2 xs = __fadd2_rn(make_float2(v[4 + p + k], v[5 + p + k]), make_float2(v[4 + p - k], v[5 + p - k]));
+      // neighbours at odd distances are not in aligned register pairs: two scalar sums
+      const float2 xs = k & 1 ? make_float2(__fadd_rn(v[4 + p + k], v[4 + p - k]), __fadd_rn(v[5 + p + k], v[5 + p - k]))
+                              : __fadd2_rn(make_float2(v[4 + p + k], v[5 + p + k]), make_float2(v[4 + p - k], v[5 + p - k]));
       const float2 ys = __fadd2_rn(h ? make_float2(yp.z, yp.w) : make_float2(yp.x, yp.y),
                                    h ? make_float2(ym.z, ym.w) : make_float2(ym.x, ym.y));
       const float2 zs = __fadd2_rn(h ? make_float2(zp.z, zp.w) : make_float2(zp.x, zp.y),
@@ -212,6 +225,66 @@ __device__ __forceinline__ void star4(const float4* Uc, const float4 (&q)[2 * R 
     }
   }
   s4[0] = s2[0].x; s4[1] = s2[0].y; s4[2] = s2[1].x; s4[3] = s2[1].y;
+}
+
+// Sampling of the source field, shared by all consumer threads of the grid:
+// it overlaps the first planes' copies.
+template <class C>
+__device__ __forceinline__ void sample_points(const PointArgs& p, int tid) {
+  const long long n = (long long)p.nshots * p.nsamp;
+  for (long long i = blockIdx.x * (long long)C::NCONS + tid; i < n; i += gridDim.x * (long long)C::NCONS) {
+    const int s = (int)(i / p.nsamp), j = (int)(i % p.nsamp);
+    const long long o = p.samp_off[i];
+    const float v = o >= 0 ? p.field_samp[s * p.samp_ss + o] : 0.f;
+    if (p.samp_out) p.samp_out[s * p.samp_out_ss + j] = v;
+    if (p.acc) p.acc[i] += (double)v * (double)p.acc_val[s * p.acc_val_ss + j];
+  }
+}
+
+// Injection into the 4 points (z, y, x ..) that this thread has just written:
+// the entry of a node that has one, all in index order of a node that has several.
+template <int MODE>
+__device__ __forceinline__ void inject_points(const TmaArgs& a, int shot, int z, int y, int x) {
+  const PointArgs& p = a.pt;
+  const int ntx = pt_tx(a.L);
+  const long long seg = ((long long)shot * a.L.nz * a.L.ny + (long long)z * a.L.ny + y) * ntx + x / PT_X;
+  const unsigned long long m = p.tiles.mask[seg];
+  const unsigned four = (unsigned)(m >> (x % PT_X)) & 15u;
+  if (!four) return;
+  const int* ent = p.tiles.ent + (long long)shot * p.ninj + p.tiles.base[seg] + __popcll(m & ((1ULL << (x % PT_X)) - 1));
+  const float* coef = p.inj_coef + (long long)shot * p.ninj;
+  const float* val = p.inj_val + shot * p.inj_val_ss;
+  const long long o = a.L.off(z, y, x);
+  float* f = a.out + shot * a.out_ss + o;
+  float* f2 = MODE == MODE_INC ? a.out2 + shot * a.out2_ss + o : nullptr;
+  int k[4];
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) k[q] = (four >> q & 1) ? ent[__popc(four & ((1u << q) - 1))] : -1;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = k[q] >= 0 ? __fmul_rn(coef[k[q]], val[k[q]]) : 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (!(four >> q & 1)) continue;
+    float u = f[q], w = MODE == MODE_INC ? f2[q] : 0.f;
+    if (k[q] >= 0) {
+      u = __fadd_rn(u, v[q]);
+      if (MODE == MODE_INC) w = __fadd_rn(w, v[q]);
+    } else {
+      const int nd = p.inj_nshared[shot];
+      const int* sh = p.inj_shared + (long long)shot * p.ninj;
+      const long long* off = p.inj_off + (long long)shot * p.ninj;
+      for (int d = 0; d < nd; ++d) {
+        const int e = sh[d];
+        if (off[e] != o + q) continue;
+        const float ve = __fmul_rn(coef[e], val[e]);
+        u = __fadd_rn(u, ve);
+        if (MODE == MODE_INC) w = __fadd_rn(w, ve);
+      }
+    }
+    f[q] = u;
+    if (MODE == MODE_INC) f2[q] = w;
+  }
 }
 
 // DAMP: the grid has an absorbing layer (the undamped instantiation carries
@@ -229,25 +302,23 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
   float* sP2 = sP1 + C::NSP * C::PFL;
   float* sG = sP2 + C::NSP * C::PFL;  // IMG only
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);
-  const uint32_t fullU = su32(bars), emptyU = fullU + 8 * C::NSU;
-  const uint32_t fullP = emptyU + 8 * C::NSU, emptyP = fullP + 8 * C::NSP;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * C::NSU + 2 * C::NSP);
+  const uint32_t full = su32(bars), empty = full + 8 * C::NSU;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * C::NSU);
 
   const int tid = threadIdx.x;
   if (tid == 0) {
     for (int s = 0; s < C::NSU; ++s) {
-      bar_init(fullU + 8 * s, 1);
-      bar_init(emptyU + 8 * s, C::NCONS / 32);
-    }
-    for (int s = 0; s < C::NSP; ++s) {
-      bar_init(fullP + 8 * s, 1);
-      bar_init(emptyP + 8 * s, C::NCONS / 32);
+      bar_init(full + 8 * s, 1);
+      bar_init(empty + 8 * s, C::NCONS / 32);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-
+  // the next sweep may be scheduled as this one's CTAs leave; its own reads and
+  // writes wait here until this grid is complete
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (tid >= C::NCONS) {
     // ------------------------------------------------------------ producer
@@ -260,29 +331,26 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
       if (nzs <= 0) continue;
       const int fu = a.f_src + sg.shot * a.fs_src, f1 = a.f_p1 + sg.shot * a.fs_p1, f2 = a.f_p2 + sg.shot * a.fs_p2;
       const int fi = a.f_img + sg.shot * a.fs_img, fg = a.f_g + sg.shot * a.fs_g;
-      for (int k = 0; k < nzs + 2 * R && ok; ++k) {
-        const int su = ku % C::NSU;
-        if (ku >= (uint32_t)C::NSU && !bar_wait(emptyU + 8 * su, ((ku / C::NSU) - 1) & 1, abort_flag, a.spin)) {
+      for (int k = 0; k < nzs + 2 * R; ++k) {
+        // the stage's last plane was the centre plane of output j - NSP (or is older): its
+        // release also frees the u_old / c2 stage of output j
+        const int j = k - 2 * R, su = ku % C::NSU;
+        if (ku >= (uint32_t)C::NSU && !bar_wait(empty + 8 * su, ((ku / C::NSU) - 1) & 1, abort_flag, a.spin)) {
           ok = false;
           break;
         }
-        bar_expect_tx(fullU + 8 * su, C::NFU * C::UBYTES);
+        const uint32_t bar = full + 8 * su;
+        bar_expect_tx(bar, C::NFU * C::UBYTES + (j >= 0 ? C::NFP * C::PBYTES : 0));
         // haloed u plane z = z0 - R + k: padded x from x0 - 4 + HX, y from y0 - R + H
-        tma4(su32(sU + su * C::UFL), &mU, sg.x0 - 4 + HX, sg.y0 - R + H, sg.z0 - R + k + H, fu, fullU + 8 * su);
+        tma4(su32(sU + su * C::UFL), &mU, sg.x0 - 4 + HX, sg.y0 - R + H, sg.z0 - R + k + H, fu, bar);
         if (C::IMG)  // the imaged field's plane, same box
-          tma4(su32(sI + su * C::UFL), &mI, sg.x0 - 4 + HX, sg.y0 - R + H, sg.z0 - R + k + H, fi, fullU + 8 * su);
+          tma4(su32(sI + su * C::UFL), &mI, sg.x0 - 4 + HX, sg.y0 - R + H, sg.z0 - R + k + H, fi, bar);
         ++ku;
-        if (k >= 2 * R) {
-          const int j = k - 2 * R;
+        if (j >= 0) {
           const int sp = kp % C::NSP;
-          if (kp >= (uint32_t)C::NSP && !bar_wait(emptyP + 8 * sp, ((kp / C::NSP) - 1) & 1, abort_flag, a.spin)) {
-            ok = false;
-            break;
-          }
-          bar_expect_tx(fullP + 8 * sp, C::NFP * C::PBYTES);
-          tma4(su32(sP1 + sp * C::PFL), &mP1, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, f1, fullP + 8 * sp);
-          tma4(su32(sP2 + sp * C::PFL), &mP2, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, f2, fullP + 8 * sp);
-          if (C::IMG) tma4(su32(sG + sp * C::PFL), &mG, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, fg, fullP + 8 * sp);
+          tma4(su32(sP1 + sp * C::PFL), &mP1, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, f1, bar);
+          tma4(su32(sP2 + sp * C::PFL), &mP2, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, f2, bar);
+          if (C::IMG) tma4(su32(sG + sp * C::PFL), &mG, sg.x0 + HX, sg.y0 + H, sg.z0 + j + H, fg, bar);
           ++kp;
         }
       }
@@ -293,14 +361,7 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
       const uint32_t uses = ku > (uint32_t)s ? (ku - 1 - s) / C::NSU + 1 : 0;
       if (uses) {
         const long long t0 = clock64();
-        while (!bar_try(fullU + 8 * s, (uses - 1) & 1) && clock64() - t0 < DEFAULT_WAIT_CYCLES) {}
-      }
-    }
-    for (int s = 0; s < C::NSP; ++s) {
-      const uint32_t uses = kp > (uint32_t)s ? (kp - 1 - s) / C::NSP + 1 : 0;
-      if (uses) {
-        const long long t0 = clock64();
-        while (!bar_try(fullP + 8 * s, (uses - 1) & 1) && clock64() - t0 < DEFAULT_WAIT_CYCLES) {}
+        while (!bar_try(full + 8 * s, (uses - 1) & 1) && clock64() - t0 < DEFAULT_WAIT_CYCLES) {}
       }
     }
     return;
@@ -309,52 +370,68 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
   // -------------------------------------------------------------- consumers
   const int tx = tid % (BX / 4), ty = tid / (BX / 4), lane = tid & 31;
   constexpr int RW = C::UW / 4;  // float4 per staged row
+  constexpr bool POINTS = MODE != MODE_IMAGE;
+  constexpr int UNROLL = (MODE != MODE_INC && !DAMP) ? 2 * R + 1 : 1;
   const float4* U4 = reinterpret_cast<const float4*>(sU);
   const float4* I4 = reinterpret_cast<const float4*>(sI);
   uint32_t ku = 0, kp = 0;
   bool ok = true;
+  if (POINTS) sample_points<C>(a.pt, tid);
   for (long long item = blockIdx.x; item < a.items && ok; item += gridDim.x) {
     const Seg sg = segment<BX, BY>(a, item);
     const int nzs = sg.z1 - sg.z0;
     if (nzs <= 0) continue;
     const int x = sg.x0 + 4 * tx, y = sg.y0 + ty;
+    // planes of this tile with injection entries: the words of the first 32 and the next
+    const unsigned* tw = nullptr;
+    unsigned tw0 = 0, tw1 = 0;
+    if (POINTS && a.pt.ninj > 0) {
+      static_assert(!POINTS || (BX == PT_X && BY == PT_Y), "point sets are by 64 x 16 columns");
+      tw = a.pt.tiles.tile + ((long long)sg.shot * a.ntx * a.nty + (long long)(sg.y0 / BY) * a.ntx + sg.x0 / BX) * pt_words(a.L);
+      tw0 = tw[sg.z0 / 32];
+      if ((sg.z1 - 1) / 32 > sg.z0 / 32) tw1 = tw[sg.z0 / 32 + 1];
+    }
     float* out = a.out + sg.shot * a.out_ss;
     float* out2 = MODE == MODE_INC ? a.out2 + sg.shot * a.out2_ss : nullptr;
     float* gout = C::IMG ? a.gout + sg.shot * a.gout_ss : nullptr;
+    const bool whole = x + 3 < a.L.nx && y < a.L.ny;
+    const long long o0 = a.L.off(sg.z0, y, x);  // this thread's points in the first plane
+    float *po = out + o0, *po2 = MODE == MODE_INC ? out2 + o0 : nullptr, *pg = C::IMG ? gout + o0 : nullptr;
     const int cidx = (ty + R) * RW + tx + 1;  // own float4 in a staged u plane
     float4 q[2 * R + 1], qi[2 * R + 1];  // qi: the imaged field's z neighbours (IMG)
     // prologue: planes z0-R .. z0+R-1 fill the queue; the first R are released
 #pragma unroll
     for (int k = 0; k < 2 * R; ++k) {
       const uint32_t kk = ku + k, s = kk % C::NSU;
-      if (!warp_wait(fullU + 8 * s, (kk / C::NSU) & 1, abort_flag, a.spin)) { ok = false; break; }
+      if (!warp_wait(full + 8 * s, (kk / C::NSU) & 1, abort_flag, a.spin)) { ok = false; break; }
       q[k] = U4[s * (C::UFL / 4) + cidx];
       if (C::IMG) qi[k] = I4[s * (C::UFL / 4) + cidx];
       if (k < R) {
         __syncwarp();
-        if (lane == 0) bar_arrive(emptyU + 8 * s);
+        if (lane == 0) bar_arrive(empty + 8 * s);
       }
     }
     // unrolled by the queue length (leapfrog and imaging sweeps): the register queue is
-    // renamed instead of shifted (32 moves per plane; 63.6 -> 59.5 us per 256^3 step)
-#pragma unroll((MODE != MODE_INC && !DAMP) ? 2 * R + 1 : 1)
+    // renamed instead of shifted (32 moves per plane; full gradient of 192 x 160 x 144,
+    // both sweeps of a step: 52.4 us against 53.3 unrolled by 1 or 3)
+    constexpr int UNROLL = (MODE != MODE_INC && !DAMP) ? 2 * R + 1 : 1;
+#pragma unroll UNROLL
     for (int j = 0; j < nzs && ok; ++j) {
       const uint32_t kc = ku + j + R, kn = ku + j + 2 * R, kq = kp + j;
       const uint32_t sc = kc % C::NSU, sn = kn % C::NSU, sp = kq % C::NSP;
-      if (!warp_wait(fullU + 8 * sn, (kn / C::NSU) & 1, abort_flag, a.spin)) { ok = false; break; }
+      if (!warp_wait(full + 8 * sn, (kn / C::NSU) & 1, abort_flag, a.spin)) { ok = false; break; }
       q[2 * R] = U4[sn * (C::UFL / 4) + cidx];
       if (C::IMG) qi[2 * R] = I4[sn * (C::UFL / 4) + cidx];
-      if (!warp_wait(fullP + 8 * sp, (kq / C::NSP) & 1, abort_flag, a.spin)) { ok = false; break; }
-      float v[12], s4[4], vi[12], si4[4];
-      star4<R, RW>(U4 + sc * (C::UFL / 4), q, cidx, a.W, v, s4);
-      if (C::IMG) star4<R, RW>(I4 + sc * (C::UFL / 4), qi, cidx, a.W, vi, si4);
-      const float4 c1 = reinterpret_cast<const float4*>(sP1 + sp * C::PFL)[ty * (BX / 4) + tx];
-      const float4 c2 = reinterpret_cast<const float4*>(sP2 + sp * C::PFL)[ty * (BX / 4) + tx];
-      const float4 g4 = C::IMG ? reinterpret_cast<const float4*>(sG + sp * C::PFL)[ty * (BX / 4) + tx] : c1;
+      float s4[4], si4[4];
+      star4<R, RW>(U4 + sc * (C::UFL / 4), q, cidx, a.W, s4);
+      if (C::IMG) star4<R, RW>(I4 + sc * (C::UFL / 4), qi, cidx, a.W, si4);
+      const int e = sp * (C::PFL / 4) + tid;
+      const float4 c1 = reinterpret_cast<const float4*>(sP1)[e], c2 = reinterpret_cast<const float4*>(sP2)[e];
+      const float4 g4 = C::IMG ? reinterpret_cast<const float4*>(sG)[e] : c1;
       float res[4], inc[4], gnew[4];
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
-        const float c = v[4 + p];
+        const float c = comp(q[R], p);
         // damping of the absorbing layer (0 outside it: the undamped expressions)
         const float ad = (DAMP && MODE != MODE_IMAGE) ? sponge_a(a.L, a.W, sg.z0 + j, y, x + p) : 0.f;
         if (MODE == MODE_STEP || MODE == MODE_STEP_IMG) {
@@ -371,26 +448,23 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
         if (C::IMG) gnew[p] = fmaf(c, si4[p], comp(g4, p));
       }
       __syncwarp();
-      if (lane == 0) {
-        bar_arrive(emptyU + 8 * sc);
-        bar_arrive(emptyP + 8 * sp);
-      }
-      if (y < a.L.ny && x < a.L.nx) {
-        const long long o = a.L.off(sg.z0 + j, y, x);
-        if (x + 3 < a.L.nx) {
-          *reinterpret_cast<float4*>(out + o) = make_float4(res[0], res[1], res[2], res[3]);
-          if (MODE == MODE_INC) *reinterpret_cast<float4*>(out2 + o) = make_float4(inc[0], inc[1], inc[2], inc[3]);
-          if (C::IMG) *reinterpret_cast<float4*>(gout + o) = make_float4(gnew[0], gnew[1], gnew[2], gnew[3]);
-        } else {
+      if (lane == 0) bar_arrive(empty + 8 * sc);
+      if (whole) {
+        *reinterpret_cast<float4*>(po) = make_float4(res[0], res[1], res[2], res[3]);
+        if (MODE == MODE_INC) *reinterpret_cast<float4*>(po2) = make_float4(inc[0], inc[1], inc[2], inc[3]);
+        if (C::IMG) *reinterpret_cast<float4*>(pg) = make_float4(gnew[0], gnew[1], gnew[2], gnew[3]);
+      } else if (y < a.L.ny) {
 #pragma unroll
-          for (int p = 0; p < 4; ++p)
-            if (x + p < a.L.nx) {
-              out[o + p] = res[p];
-              if (MODE == MODE_INC) out2[o + p] = inc[p];
-              if (C::IMG) gout[o + p] = gnew[p];
-            }
-        }
+        for (int p = 0; p < 4; ++p)
+          if (x + p < a.L.nx) {
+            po[p] = res[p];
+            if (MODE == MODE_INC) po2[p] = inc[p];
+            if (C::IMG) pg[p] = gnew[p];
+          }
       }
+      po += a.L.plane;
+      if (MODE == MODE_INC) po2 += a.L.plane;
+      if (C::IMG) pg += a.L.plane;
 #pragma unroll
       for (int k = 0; k < 2 * R; ++k) {
         q[k] = q[k + 1];
@@ -401,10 +475,19 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
     // the last R planes were only queue heads: release them
     for (int k = nzs + R; k < nzs + 2 * R; ++k) {
       __syncwarp();
-      if (lane == 0) bar_arrive(emptyU + 8 * ((ku + k) % C::NSU));
+      if (lane == 0) bar_arrive(empty + 8 * ((ku + k) % C::NSU));
     }
     ku += nzs + 2 * R;
     kp += nzs;
+    if (POINTS && tw && x < a.L.nx && y < a.L.ny)
+      for (int w = sg.z0 / 32; w <= (sg.z1 - 1) / 32; ++w) {
+        unsigned m = w == sg.z0 / 32 ? tw0 : (w == sg.z0 / 32 + 1 ? tw1 : tw[w]);
+        for (; m; m &= m - 1) {
+          const int z = 32 * w + __ffs(m) - 1;
+          if (z < sg.z0 || z >= sg.z1) continue;
+          inject_points<MODE>(a, sg.shot, z, y, x);
+        }
+      }
   }
   if (!ok && lane == 0) atomicOr(a.err, 1);
 }
@@ -483,8 +566,17 @@ cudaError_t launch_k(const CUtensorMap& mU, const CUtensorMap& m1, const CUtenso
                      const CUtensorMap& mG, const TmaArgs& t, long long blocks, cudaStream_t s) {
   const cudaError_t e = smem_limit_once<sweep3d_tma<R, MODE, C, DAMP>>((int)C::SMEM);
   if (e != cudaSuccess) return e;
-  sweep3d_tma<R, MODE, C, DAMP><<<(unsigned)blocks, C::NTHREADS, C::SMEM, s>>>(mU, m1, m2, mI, mG, t);
-  return cudaGetLastError();
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;  // the kernel waits for the one before it by itself
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(C::NTHREADS);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, sweep3d_tma<R, MODE, C, DAMP>, mU, m1, m2, mI, mG, t);
 }
 
 template <int R, int MODE, class C>
@@ -517,24 +609,30 @@ cudaError_t launch_c(const Layout& L, const Weights& W, const StencilArgs& a, cu
   t.nshots = a.nshots;
   t.ntx = (L.nx + BX - 1) / BX;
   t.nty = (L.ny + BY - 1) / BY;
+  t.pt = a.pt;
   t.err = err;
   t.spin = wait_limit_cycles();
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // z chunks per tile column: the fewest that fill the CTA slots (2 per SM)
-  // to at least 90 % over whole waves, else as many as keep one wave busy
-  // (256^3: 64 columns x 9 chunks on 304 slots ran 3 % faster than 4 chunks,
-  // which left 48 slots idle)
+  // z chunks per tile column: a CTA's time is, in planes, chunk + 10 for its
+  // first item (2R planes of halo, the launch and the first copies' latency)
+  // and chunk + 2R for each further one, whose first planes are prefetched.
+  // Measured per plane of this count, 2 to 30 chunks, one to four waves:
+  // 0.41-0.43 us (131 x 119 x 107 x 2, order 4), 0.42-0.54 (192 x 160 x 144,
+  // order 8), 0.60-0.66 (256^3, order 8: HBM).  For every number of waves the
+  // shortest chunks that it holds; the best of eight.
   const int occ = (int)std::max<size_t>(1, std::min<size_t>(2, (228 * 1024) / (C::SMEM + 1024)));
   const long long cols = (long long)t.ntx * t.nty * a.nshots, slots = (long long)occ * sms;
-  const int zmax = std::max(1, L.nz / (3 * R));
-  t.nzc = (int)std::max<long long>(1, std::min<long long>(slots / cols, std::max(1, L.nz / (4 * R))));
-  for (int c = (int)std::max<long long>(1, (slots + cols - 1) / cols); c <= zmax; ++c) {
-    const long long items = cols * c, waves = (items + slots - 1) / slots;
-    if (items * 10 >= waves * slots * 9 && waves <= 3) {
+  long long best = 0;
+  const long long w0 = (cols + slots - 1) / slots;
+  for (long long w = w0; w < w0 + 8; ++w) {
+    const int c = (int)std::min<long long>(w * slots / cols, std::max(1, L.nz / 2));
+    const int chunk = (L.nz + c - 1) / c;
+    const long long cost = chunk + 10 + (w - 1) * (chunk + 2 * R);
+    if (w == w0 || cost < best) {
+      best = cost;
       t.nzc = c;
-      break;
     }
   }
   t.zchunk = (L.nz + t.nzc - 1) / t.nzc;
