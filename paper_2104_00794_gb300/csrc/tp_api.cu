@@ -136,6 +136,12 @@ Weights stencil_weights(int order) {
 
 namespace {
 
+// Levels of the adjoint wavefield that the full-storage 2-D gradient forms per
+// launch and then images in one pass over their history.  Gradient of 397 x 401,
+// 4 shots, order 8, us per level: 16 levels 10.5, 32 10.0, 64 9.7 (for twice the
+// ring); a launch per step, its points and its image 31.1.
+constexpr int FULL_WINDOW = 32;
+
 struct Plan {
   int op = 0;
   Layout L{};
@@ -303,7 +309,11 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
     case TP_OP_GRADIENT_FULL:
       P->nf = (long long)P->nt * ns;
       P->o_f = take(cur, (size_t)P->nf * fb);   // forward history, levels 0..nt-1
-      P->o_P = take(cur, (size_t)3 * ns * fb);  // adjoint levels
+      // adjoint levels: three, or (persistent 2-D path) a window of them and their values at the sources
+      P->T = P->c2d ? std::max(1, std::min(FULL_WINDOW, P->nt - 2)) : 1;
+      P->S = P->T + 2;
+      P->o_P = take(cur, (size_t)P->S * ns * fb);
+      if (P->c2d) P->o_Q = take(cur, (size_t)ns * P->nt * P->nsrc * sizeof(float));
       P->o_d = take(cur, (size_t)ns * P->nt * P->nrec * sizeof(float));
       P->o_gacc = take(cur, (size_t)ns * fb);
       P->o_sacc = take(cur, (size_t)ns * P->nsrc * sizeof(double));
@@ -975,18 +985,19 @@ tp_status tp_gradient_full(const tp_grid* grid, const tp_geom* geom, const float
   const size_t fb = (size_t)P.L.field * sizeof(float);
   const int nt = P.nt;
   TRY(cudaMemsetAsync(c.at<float>(P.o_f), 0, (size_t)P.nf * fb, c.st));
-  TRY(cudaMemsetAsync(c.at<float>(P.o_P), 0, (size_t)3 * P.nshots * fb, c.st));
+  TRY(cudaMemsetAsync(c.at<float>(P.o_P), 0, (size_t)P.S * P.nshots * fb, c.st));
   TRY(cudaMemsetAsync(c.at<float>(P.o_gacc), 0, (size_t)P.nshots * fb, c.st));
   TRY(cudaMemsetAsync(c.at<double>(P.o_sacc), 0, (size_t)P.nshots * P.nsrc * sizeof(double), c.st));
   float* d = c.at<float>(P.o_d);
   TRY(cudaMemsetAsync(d, 0, (size_t)P.nshots * nt * P.nrec * sizeof(float), c.st));
-  const Fam fh{P.o_f, (int)P.nf, nt}, fl{P.o_P, 3 * P.nshots, 3}, fG{P.o_gacc, P.nshots, 1};
+  const Fam fh{P.o_f, (int)P.nf, nt}, fl{P.o_P, P.S * P.nshots, P.S}, fG{P.o_gacc, P.nshots, 1};
   auto hist = [](int t) { return t; };
   TRYS(forward_loop(c, fh, hist, wavelet, d, [](int) { return TP_OK; }, [](int) { return false; }));
   TRYS(misfit_and_residual(c, d, d_obs, misfit));
   // adjoint with the imaging condition of Eq. 3 in its stencil form:
   // gacc_s += lambda_s[j] * S(u_s[j-1])   (udd[j] = v^2 (L u[j-1] + S^T q[j-1]))
-  auto lam = [](int k) { return k % 3; };
+  const int S = P.S;
+  auto lam = [S](int k) { return k % S; };
   if (P.L.ndim == 3 && P.form == TP_FORM_LEVELS) {
     // 3-D: in the sweep of the step that forms lambda[j], whose source field
     // lambda[j+1] is complete: the terms j+1 = nt .. 3 in the same order and
@@ -1005,6 +1016,18 @@ tp_status tp_gradient_full(const tp_grid* grid, const tp_geom* geom, const float
     };
     TRYS(adjoint_loop(c, fl, lam, d, nullptr, c.at<double>(P.o_sacc), wavelet, [](int) { return TP_OK; },
                       [](int) { return true; }, fused));
+  } else if (P.c2d) {
+    // windows of T levels on the persistent path, then their terms in one pass, in the same order
+    auto closes = adj_window_closes(nt, P.T);
+    auto imaging = [&](int j) -> tp_status {
+      if (!closes(j)) return TP_OK;
+      const int top = nt - 1 - ((nt - 1 - j) / P.T) * P.T;
+      TRY(launch_image_window2d(P.L, P.W, c.ptr(fh, 0), c.ss(fh), c.ptr(fl, 0), c.ss(fl), S, top, top - j + 1,
+                                c.ptr(fG, 0), c.ss(fG), P.nshots, c.st));
+      return TP_OK;
+    };
+    TRYS(adjoint_loop(c, fl, lam, d, c.at<float>(P.o_Q), nullptr, nullptr, imaging, closes));
+    TRY(launch_source_dot(c.at<float>(P.o_Q), wavelet, nt, P.nsrc, P.nshots, c.at<double>(P.o_sacc), c.st));
   } else {
     auto imaging = [&](int j) -> tp_status {
       StencilArgs a{c.ref(fh, j - 1), c.ref(fl, lam(j)), c.ref(fG, 0), c.ptr(fG, 0), c.ss(fG), P.nshots};

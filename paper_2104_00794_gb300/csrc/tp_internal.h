@@ -152,6 +152,11 @@ struct StencilArgs {
 };
 cudaError_t launch_stencil(int mode, const Layout& L, const Weights& W, const StencilArgs& a,
                            cudaStream_t s, int* err);
+// 2-D: g += lam[j] * S(u[j - 1]) for the levels j = top .. top - nlev + 1 in
+// this order (level t of u: field t of its shot, of lam: field t mod nslots)
+cudaError_t launch_image_window2d(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
+                                  long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
+                                  cudaStream_t s);
 // 4-D TMA map over a family of `nfields` consecutive padded fields of `esize`
 // bytes per value (4: fp32, 2: bf16): dims (px, py, pz, nfields), box
 // (box_x, box_y, 1, box_fields), no swizzle; encoded once per distinct key.
@@ -268,6 +273,9 @@ cudaError_t launch_image(const Layout& L, int order, float h, int cond, const fl
 // qbar[s][k][i] = sum_{j=jlo}^{jhi} Q[s][j + qshift][i] * q[s][j][k]
 cudaError_t launch_qbar(const float* Q, int nt, int r, const float* wav, int nsrc, int nshots,
                         int jlo, int jhi, int qshift, float* qbar, cudaStream_t s);
+// acc[s][k] = sum_{j=1}^{nt-2} q[s][j][k] * wav[s][j][k]
+cudaError_t launch_source_dot(const float* q, const float* wav, int nt, int nsrc, int nshots, double* acc,
+                              cudaStream_t s);
 // grad[src[s][k]] += -scale * vel^2 * (probed: sum_i qbar[s][k][i] vbar[s][i][off]; full: srcacc[s][k])
 // serial in a fixed order (deterministic when sources share a node)
 cudaError_t launch_source_term(const Layout& L, const float* vel, const int64_t* src_dense,

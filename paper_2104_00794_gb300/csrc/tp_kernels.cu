@@ -339,6 +339,17 @@ __global__ void qbar_kernel(const float* __restrict__ Q, int nt, int r, const fl
   qbar[e] = (float)acc;
 }
 
+__global__ void __launch_bounds__(RED_THREADS) source_dot_kernel(const float* __restrict__ q,
+                                                                 const float* __restrict__ wav, int nt, int nsrc,
+                                                                 double* __restrict__ acc) {
+  const long long e = blockIdx.x, o = e / nsrc * ((long long)nt * nsrc) + e % nsrc;
+  double v = 0.0;
+  for (int j = 1 + threadIdx.x; j <= nt - 2; j += RED_THREADS)
+    v += (double)q[o + (long long)j * nsrc] * (double)wav[o + (long long)j * nsrc];
+  v = block_sum(v);
+  if (threadIdx.x == 0) acc[e] = v;
+}
+
 // value of accumulator i at element o of one shot's accumulator block
 __device__ __forceinline__ float acc_value(const void* P, int acc, int r, int i, long long field, long long o) {
   if (acc == 0) return static_cast<const float*>(P)[(long long)i * field + o];
@@ -510,6 +521,14 @@ cudaError_t launch_qbar(const float* Q, int nt, int r, const float* wav, int nsr
   prof_before(5, s);
   const int n = nshots * nsrc * r;
   qbar_kernel<<<(n + 127) / 128, 128, 0, s>>>(Q, nt, r, wav, nsrc, nshots, jlo, jhi, qshift, qbar);
+  prof_after(5, s);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_source_dot(const float* q, const float* wav, int nt, int nsrc, int nshots, double* acc,
+                              cudaStream_t s) {
+  prof_before(5, s);
+  source_dot_kernel<<<(unsigned)((long long)nshots * nsrc), RED_THREADS, 0, s>>>(q, wav, nt, nsrc, acc);
   prof_after(5, s);
   return cudaGetLastError();
 }

@@ -156,6 +156,78 @@ sweep2d(Layout L, Weights W, PlainArgs a, int bz, int nzc, int nxt, int nwarps) 
   }
 }
 
+// The imaging terms of a window of levels (2-D): g += lam[j] * S(u[j - 1]), j =
+// top .. top - nlev + 1 in this order, the additions of a sweep per level
+// (MODE_IMAGE) in one launch.  A warp keeps NB rows of 128 points of g in
+// registers over the window; a level's loads are independent of the last
+// one's sums, and the rows that neighbouring warps of a CTA share hit in L1.
+// 12.1 us per level as sweeps of their own (397 x 401 x 4 shots), 1.7 in windows
+// of 32: L1 bandwidth and latency.  NB = 2: 8 loads of 16 B a row of a lane and
+// 16 warps an SM there; full gradient 10.0 us a level, with 4 rows (6 loads, 8
+// warps) 10.5, with 1 11.1, with 8 12.4.
+// Level j of u is field j, of lam field j mod nslots of a shot.
+template <int R, int NB>
+__global__ void __launch_bounds__(32 * W2)
+image2d_window(Layout L, Weights W, const float* __restrict__ u, long long u_ss, const float* __restrict__ lam,
+               long long lam_ss, int nslots, int top, int nlev, float* __restrict__ g, long long g_ss, int nxt,
+               int nzc, int nwarps) {
+  const int gw = blockIdx.x * W2 + threadIdx.y, lane = threadIdx.x;
+  if (gw >= nwarps) return;
+  const int zc = gw % nzc, xt = gw / nzc % nxt, shot = gw / (nzc * nxt);
+  const int x = xt * 128 + 4 * lane, zb = zc * NB;
+  const long long pl = L.px, col = x + HX + (long long)H * pl;
+  // rows beyond the bottom halo are only read for rows that are not stored
+  auto row = [&](int z) { return col + (long long)min(z, L.nz + H - 1) * pl; };
+  u += shot * u_ss;
+  lam += shot * lam_ss;
+  g += shot * g_ss;
+  float4 acc[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) acc[b] = *reinterpret_cast<const float4*>(g + row(zb + b));
+  const float2 m4 = make_float2(-4.f, -4.f);
+  for (int i = 0; i < nlev; ++i) {
+    const int j = top - i;
+    const float* us = u + (j - 1) * L.field;
+    const float* ls = lam + (j % nslots) * L.field;
+    float4 c[NB + 2 * R], xl[NB], xr[NB], l[NB];
+#pragma unroll
+    for (int b = 0; b < NB + 2 * R; ++b) c[b] = ld4(us, row(zb - R + b));
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      xl[b] = ld4(us, row(zb + b) - 4);
+      xr[b] = ld4(us, row(zb + b) + 4);
+      l[b] = ld4(ls, row(zb + b));
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const float4 xc = c[b + R];
+      const float v[12] = {xl[b].x, xl[b].y, xl[b].z, xl[b].w, xc.x, xc.y, xc.z, xc.w, xr[b].x, xr[b].y, xr[b].z, xr[b].w};
+      float2 s2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+      for (int k = 1; k <= R; ++k) {
+        const float4 zp = c[b + R + k], zm = c[b + R - k];
+        const float2 wk = make_float2(W.w[k], W.w[k]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int p = 2 * h;
+          const float2 ctr = make_float2(v[4 + p], v[5 + p]);
+          const float2 xs = __fadd2_rn(make_float2(v[4 + p + k], v[5 + p + k]), make_float2(v[4 + p - k], v[5 + p - k]));
+          const float2 zs = __fadd2_rn(h ? make_float2(zp.z, zp.w) : make_float2(zp.x, zp.y),
+                                       h ? make_float2(zm.z, zm.w) : make_float2(zm.x, zm.y));
+          s2[h] = __ffma2_rn(wk, __ffma2_rn(m4, ctr, __fadd2_rn(xs, zs)), s2[h]);
+        }
+      }
+      acc[b].x = fmaf(l[b].x, s2[0].x, acc[b].x);
+      acc[b].y = fmaf(l[b].y, s2[0].y, acc[b].y);
+      acc[b].z = fmaf(l[b].z, s2[1].x, acc[b].z);
+      acc[b].w = fmaf(l[b].w, s2[1].y, acc[b].w);
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+    if (zb + b < L.nz && x < L.nx) store_masked(g, row(zb + b), acc[b], x, L.nx);
+}
+
 // SM count of the current device, cached per device (thread-safe)
 int num_sms() {
   static std::atomic<int> cache[64];
@@ -186,7 +258,28 @@ cudaError_t launch2d(const Layout& L, const Weights& W, const PlainArgs& a, cuda
   return cudaGetLastError();
 }
 
+template <int R>
+cudaError_t image_window(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
+                         long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
+                         cudaStream_t s) {
+  constexpr int NB = 2;
+  const int nxt = (L.nx + 127) / 128, nzc = (L.nz + NB - 1) / NB, nwarps = nxt * nzc * nshots;
+  image2d_window<R, NB><<<(nwarps + W2 - 1) / W2, dim3(32, W2), 0, s>>>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g,
+                                                                        g_ss, nxt, nzc, nwarps);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+cudaError_t launch_image_window2d(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
+                                  long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
+                                  cudaStream_t s) {
+  prof_before(1, s);
+  const cudaError_t e = W.R == 4 ? image_window<4>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g, g_ss, nshots, s)
+                                 : image_window<2>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g, g_ss, nshots, s);
+  prof_after(1, s);
+  return e;
+}
 
 cudaError_t launch_sweep3d_tma(int mode, const Layout& L, const Weights& W, const StencilArgs& a, cudaStream_t s,
                                int* err);
