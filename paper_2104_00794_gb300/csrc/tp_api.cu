@@ -839,11 +839,16 @@ tp_status probed_backward_impl(const Ctx& c, const tp_grid* grid, const tp_geom*
     // the state's accumulators and the workspace's vbar as field families
     const FieldRef fPr{static_cast<const float*>(Pacc), (int)accf, 0, r};
     const Fam fV{vo, (int)accf, r};
-    for (int i = 0; i < r; ++i) {
-      FieldRef pi = fPr;
-      pi.f0 = i;
-      StencilArgs a{pi, c.ref(fV, i), c.ref(fG, 0), c.ptr(fG, 0), c.ss(fG), P.nshots};
-      TRY(launch_stencil(MODE_IMAGE, P.L, P.W, a, c.st, c.err()));
+    if (P.L.ndim == 2) {  // all probes in one launch, the sums of the loop below
+      TRY(launch_image_window2d(P.L, P.W, static_cast<const float*>(Pacc), P.acc_elems, c.ptr(fV, 0), P.acc_elems, r, 0,
+                                1, 0, r, c.ptr(fG, 0), c.ss(fG), P.nshots, c.st));
+    } else {
+      for (int i = 0; i < r; ++i) {
+        FieldRef pi = fPr;
+        pi.f0 = i;
+        StencilArgs a{pi, c.ref(fV, i), c.ref(fG, 0), c.ptr(fG, 0), c.ss(fG), P.nshots};
+        TRY(launch_stencil(MODE_IMAGE, P.L, P.W, a, c.st, c.err()));
+      }
     }
   } else {
     // bf16 storage: fp32 copies of P_i and V_i (per shot) feed the same sweep
@@ -1022,7 +1027,7 @@ tp_status tp_gradient_full(const tp_grid* grid, const tp_geom* geom, const float
     auto imaging = [&](int j) -> tp_status {
       if (!closes(j)) return TP_OK;
       const int top = nt - 1 - ((nt - 1 - j) / P.T) * P.T;
-      TRY(launch_image_window2d(P.L, P.W, c.ptr(fh, 0), c.ss(fh), c.ptr(fl, 0), c.ss(fl), S, top, top - j + 1,
+      TRY(launch_image_window2d(P.L, P.W, c.ptr(fh, 0), c.ss(fh), c.ptr(fl, 0), c.ss(fl), S, top, -1, -1, top - j + 1,
                                 c.ptr(fG, 0), c.ss(fG), P.nshots, c.st));
       return TP_OK;
     };

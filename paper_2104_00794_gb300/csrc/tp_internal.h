@@ -152,11 +152,11 @@ struct StencilArgs {
 };
 cudaError_t launch_stencil(int mode, const Layout& L, const Weights& W, const StencilArgs& a,
                            cudaStream_t s, int* err);
-// 2-D: g += lam[j] * S(u[j - 1]) for the levels j = top .. top - nlev + 1 in
-// this order (level t of u: field t of its shot, of lam: field t mod nslots)
+// 2-D: g += lam[j] * S(u[j + shift]) for the nlev levels j = first, first + dir, ..
+// in this order (level t of u: field t of its shot, of lam: field t mod nslots)
 cudaError_t launch_image_window2d(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
-                                  long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
-                                  cudaStream_t s);
+                                  long long lam_ss, int nslots, int first, int dir, int shift, int nlev, float* g,
+                                  long long g_ss, int nshots, cudaStream_t s);
 // 4-D TMA map over a family of `nfields` consecutive padded fields of `esize`
 // bytes per value (4: fp32, 2: bf16): dims (px, py, pz, nfields), box
 // (box_x, box_y, 1, box_fields), no swizzle; encoded once per distinct key.

@@ -328,15 +328,29 @@ __global__ void source_into_acc_kernel(const long long* __restrict__ soff, const
     }
 }
 
-__global__ void qbar_kernel(const float* __restrict__ Q, int nt, int r, const float* __restrict__ wav, int nsrc,
-                            int nshots, int jlo, int jhi, int qshift, float* __restrict__ qbar) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nshots * nsrc * r) return;
-  const int s = e / (nsrc * r), k = (e / r) % nsrc, i = e % r;
+// One block per shot, source and rp (a power of two, at most 32) probes: the
+// time levels are shared by the threads of a probe, their fp64 sums added in
+// order.  (A thread per probe over all levels took 0.9 ms for 3000 of them, the
+// latency of its loads.)
+constexpr int QBAR_THREADS = 512;
+__global__ void __launch_bounds__(QBAR_THREADS) qbar_kernel(const float* __restrict__ Q, int nt, int r, int rp,
+                                                            const float* __restrict__ wav, int nsrc, int jlo, int jhi,
+                                                            int qshift, float* __restrict__ qbar) {
+  __shared__ double part[QBAR_THREADS];
+  const int s = blockIdx.x / nsrc, k = blockIdx.x % nsrc, tid = threadIdx.x;
+  const int i = blockIdx.y * rp + tid % rp, g = tid / rp, ng = QBAR_THREADS / rp;
   double acc = 0.0;
-  for (int j = jlo; j <= jhi; ++j)
-    acc += (double)Q[((long long)s * nt + j + qshift) * r + i] * (double)wav[((long long)s * nt + j) * nsrc + k];
-  qbar[e] = (float)acc;
+  if (i < r) {
+#pragma unroll 8
+    for (int j = jlo + g; j <= jhi; j += ng)
+      acc += (double)Q[((long long)s * nt + j + qshift) * r + i] * (double)wav[((long long)s * nt + j) * nsrc + k];
+  }
+  part[tid] = acc;
+  __syncthreads();
+  if (g == 0 && i < r) {
+    for (int q = 1; q < ng; ++q) acc += part[q * rp + tid];
+    qbar[(long long)blockIdx.x * r + i] = (float)acc;
+  }
 }
 
 __global__ void __launch_bounds__(RED_THREADS) source_dot_kernel(const float* __restrict__ q,
@@ -519,8 +533,10 @@ cudaError_t launch_finish_grad(const Layout& L, const float* vel, const float* g
 cudaError_t launch_qbar(const float* Q, int nt, int r, const float* wav, int nsrc, int nshots, int jlo, int jhi,
                         int qshift, float* qbar, cudaStream_t s) {
   prof_before(5, s);
-  const int n = nshots * nsrc * r;
-  qbar_kernel<<<(n + 127) / 128, 128, 0, s>>>(Q, nt, r, wav, nsrc, nshots, jlo, jhi, qshift, qbar);
+  int rp = 1;
+  while (rp < r && rp < 32) rp *= 2;
+  qbar_kernel<<<dim3((unsigned)((long long)nshots * nsrc), (r + rp - 1) / rp), QBAR_THREADS, 0, s>>>(
+      Q, nt, r, rp, wav, nsrc, jlo, jhi, qshift, qbar);
   prof_after(5, s);
   return cudaGetLastError();
 }

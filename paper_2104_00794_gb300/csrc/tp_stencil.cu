@@ -156,21 +156,22 @@ sweep2d(Layout L, Weights W, PlainArgs a, int bz, int nzc, int nxt, int nwarps) 
   }
 }
 
-// The imaging terms of a window of levels (2-D): g += lam[j] * S(u[j - 1]), j =
-// top .. top - nlev + 1 in this order, the additions of a sweep per level
-// (MODE_IMAGE) in one launch.  A warp keeps NB rows of 128 points of g in
+// The imaging terms of a window of levels (2-D): g += lam[j] * S(u[j + shift]), j =
+// first, first + dir, .. (nlev levels) in this order, the additions of a sweep per
+// level (MODE_IMAGE) in one launch.  A warp keeps NB rows of 128 points of g in
 // registers over the window; a level's loads are independent of the last
 // one's sums, and the rows that neighbouring warps of a CTA share hit in L1.
 // 12.1 us per level as sweeps of their own (397 x 401 x 4 shots), 1.7 in windows
 // of 32: L1 bandwidth and latency.  NB = 2: 8 loads of 16 B a row of a lane and
 // 16 warps an SM there; full gradient 10.0 us a level, with 4 rows (6 loads, 8
 // warps) 10.5, with 1 11.1, with 8 12.4.
-// Level j of u is field j, of lam field j mod nslots of a shot.
+// Level j of u is field j, of lam field j mod nslots of a shot.  The combination
+// of r probes is the same sum over them.
 template <int R, int NB>
 __global__ void __launch_bounds__(32 * W2)
 image2d_window(Layout L, Weights W, const float* __restrict__ u, long long u_ss, const float* __restrict__ lam,
-               long long lam_ss, int nslots, int top, int nlev, float* __restrict__ g, long long g_ss, int nxt,
-               int nzc, int nwarps) {
+               long long lam_ss, int nslots, int first, int dir, int shift, int nlev, float* __restrict__ g,
+               long long g_ss, int nxt, int nzc, int nwarps) {
   const int gw = blockIdx.x * W2 + threadIdx.y, lane = threadIdx.x;
   if (gw >= nwarps) return;
   const int zc = gw % nzc, xt = gw / nzc % nxt, shot = gw / (nzc * nxt);
@@ -186,8 +187,8 @@ image2d_window(Layout L, Weights W, const float* __restrict__ u, long long u_ss,
   for (int b = 0; b < NB; ++b) acc[b] = *reinterpret_cast<const float4*>(g + row(zb + b));
   const float2 m4 = make_float2(-4.f, -4.f);
   for (int i = 0; i < nlev; ++i) {
-    const int j = top - i;
-    const float* us = u + (j - 1) * L.field;
+    const int j = first + dir * i;
+    const float* us = u + (j + shift) * L.field;
     const float* ls = lam + (j % nslots) * L.field;
     float4 c[NB + 2 * R], xl[NB], xr[NB], l[NB];
 #pragma unroll
@@ -260,23 +261,23 @@ cudaError_t launch2d(const Layout& L, const Weights& W, const PlainArgs& a, cuda
 
 template <int R>
 cudaError_t image_window(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
-                         long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
-                         cudaStream_t s) {
+                         long long lam_ss, int nslots, int first, int dir, int shift, int nlev, float* g,
+                         long long g_ss, int nshots, cudaStream_t s) {
   constexpr int NB = 2;
   const int nxt = (L.nx + 127) / 128, nzc = (L.nz + NB - 1) / NB, nwarps = nxt * nzc * nshots;
-  image2d_window<R, NB><<<(nwarps + W2 - 1) / W2, dim3(32, W2), 0, s>>>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g,
-                                                                        g_ss, nxt, nzc, nwarps);
+  image2d_window<R, NB><<<(nwarps + W2 - 1) / W2, dim3(32, W2), 0, s>>>(
+      L, W, u, u_ss, lam, lam_ss, nslots, first, dir, shift, nlev, g, g_ss, nxt, nzc, nwarps);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_image_window2d(const Layout& L, const Weights& W, const float* u, long long u_ss, const float* lam,
-                                  long long lam_ss, int nslots, int top, int nlev, float* g, long long g_ss, int nshots,
-                                  cudaStream_t s) {
+                                  long long lam_ss, int nslots, int first, int dir, int shift, int nlev, float* g,
+                                  long long g_ss, int nshots, cudaStream_t s) {
   prof_before(1, s);
-  const cudaError_t e = W.R == 4 ? image_window<4>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g, g_ss, nshots, s)
-                                 : image_window<2>(L, W, u, u_ss, lam, lam_ss, nslots, top, nlev, g, g_ss, nshots, s);
+  const auto run = W.R == 4 ? image_window<4> : image_window<2>;
+  const cudaError_t e = run(L, W, u, u_ss, lam, lam_ss, nslots, first, dir, shift, nlev, g, g_ss, nshots, s);
   prof_after(1, s);
   return e;
 }
