@@ -155,6 +155,15 @@ typedef struct {
  * the reason in tp_last_error().  No device work. */
 tp_status tp_form_supported(const tp_grid* grid, const tp_geom* geom);
 
+/* How calls on this grid and batch (only the counts of geom are read) are
+ * stepped, forward or adjoint; a diagnostic.  plan[0]: 0 a launch per step, 1
+ * bands of all shots in one cooperative grid, 2 a thread-block cluster per shot;
+ * then for 1 and 2: CTAs per shot, grid rows per CTA, rows per march, shots at
+ * once, whether the coefficients are in shared memory.  Planned for the current
+ * device, or for a GB300 where there is none; no device work.  Errors:
+ * TP_ERR_ARG as tp_form_supported. */
+tp_status tp_sweep2d_plan(const tp_grid* grid, const tp_geom* geom, int adjoint, int plan[6]);
+
 /* Bytes of device workspace that `op` needs (0 on invalid arguments; see
  * tp_last_error).  `probe` is read only for the probed ops.  The workspace
  * must be 256-byte aligned. */

@@ -635,6 +635,19 @@ tp_status tp_form_supported(const tp_grid* grid, const tp_geom* geom) {
   return TP_OK;
 }
 
+tp_status tp_sweep2d_plan(const tp_grid* grid, const tp_geom* geom, int adjoint, int plan[6]) {
+  if (!plan) return fail(TP_ERR_ARG, "plan is NULL");
+  TRYS(tp_form_supported(grid, geom));
+  for (int i = 0; i < 6; ++i) plan[i] = 0;
+  const Layout L = make_layout(grid->ndim, grid->nx, grid->ny, grid->nz);
+  Weights W = stencil_weights(grid->order);
+  W.sw = grid->sponge_eta > 0.f ? grid->sponge : 0;
+  const bool comp = grid->form == TP_FORM_COMPENSATED;
+  if (comp || (grid->form == TP_FORM_LEVELS && persist2d_fits(L, W, geom->nshots, geom->nsrc, geom->nrec)))
+    plan2d(L, W, comp && !adjoint, geom->nshots, adjoint ? geom->nrec : geom->nsrc, adjoint ? geom->nsrc : geom->nrec, plan);
+  return TP_OK;
+}
+
 size_t tp_workspace_bytes(int op, const tp_grid* grid, const tp_geom* geom, const tp_probe* probe) {
   Plan P;
   if (make_plan(op, grid, geom, probe, &P) != TP_OK) return 0;

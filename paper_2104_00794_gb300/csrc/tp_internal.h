@@ -199,6 +199,8 @@ bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int
 // bands of the whole GPU
 bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec);
 size_t edge2d_bytes(const Layout& L, const Weights& W);
+// the split that launch_cluster2d takes on the current device (tp_sweep2d_plan)
+void plan2d(const Layout& L, const Weights& W, bool comp, int nshots, int ninj, int nsamp, int plan[6]);
 
 // ---------------------------------------------------------------- probe GEMM
 // P[s][i][x] += sum_{k < nlev} ring[s][(level0 + k) mod nslots][x] * Q[s][level0 + k + qshift][i]

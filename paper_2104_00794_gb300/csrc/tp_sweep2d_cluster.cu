@@ -328,9 +328,16 @@ __device__ __forceinline__ void row4(const Weights& W, const float4* u, Low low,
 // unrolled, so that the queue moves once per block).  The band's rpc rows are a
 // multiple of N; rows past the grid and columns past nx have c2 = 0 and stay
 // zero, so that no row and no column is guarded.
+// LEAN (clusters without c2 in shared memory, for wide grids): the levels alone
+// fill the shared memory.  c2 comes from global memory, nothing is kept per
+// unit, all entries are added after the march, and the last chunk of a band
+// has as many rows as are left.  Compensated step, order 8: 1800 x 100 9.3 us,
+// 2001 x 101 x 8 shots 11.5 us (8.9 and 17.7 us when a cluster kept c2 in global
+// memory and guarded every row).
 template <int R, int MODE, bool BAND, int N, bool C2S>
 __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
-  constexpr bool COMP = MODE == C2_COMP, DAMP = MODE == C2_DAMP;
+  constexpr bool COMP = MODE == C2_COMP, DAMP = MODE == C2_DAMP, LEAN = !BAND && !C2S;
+  static_assert(!LEAN || (!DAMP && N <= 4), "a lean march is one block of rows without a layer");
   constexpr int PER = C2_MAXLIST / C2_THREADS;  // list entries per thread
   const int tid = threadIdx.x;
   const int C = a.C, rank = blockIdx.x % C, cid = blockIdx.x / C, ncl = gridDim.x / C;
@@ -338,7 +345,8 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   const int nz = a.L.nz, nx = a.L.nx, px = a.L.px;
   const int z0 = rank * rpc;
   const int nrow = min(rpc, nz - z0);  // rows of the grid that this CTA owns (>= 1)
-  const int nch = rpc / N, units = nch * nx4;
+  const int nch = LEAN ? (rpc + N - 1) / N : rpc / N, units = nch * nx4;
+  const int ntab = LEAN ? 0 : units;  // units with entries in the tables below
 
   // shared memory: both levels of the band, a zero row (clusters), the low
   // parts of both levels (COMP), c2, the band's injection and sampling
@@ -375,11 +383,11 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   //          offsets for parity 0), chain's first entry | march row of the line
   //          << 16, column
   int4* const ua_ = reinterpret_cast<int4*>(ival + 2 * vstep);
-  int4* const ub_ = ua_ + units;
-  ushort4* const uline = reinterpret_cast<ushort4*>(ub_ + units);
-  uint16_t* const tl = reinterpret_cast<uint16_t*>(uline + units);  // last entry of a unit (set-up)
-  uint16_t* const nxt = tl + (units + 1) / 2 * 2;                // next entry of the same unit; LEAD: entries of its node
-  int* const cnt = reinterpret_cast<int*>(nxt + (units + 1) / 2 % 2 * 2 + a.capi);  // [0] injection, [1] sampling entries, [3] LEAD used, [4 ..] per-warp counts
+  int4* const ub_ = ua_ + ntab;
+  ushort4* const uline = reinterpret_cast<ushort4*>(ub_ + ntab);
+  uint16_t* const tl = reinterpret_cast<uint16_t*>(uline + ntab);  // last entry of a unit (set-up)
+  uint16_t* const nxt = tl + (ntab + 1) / 2 * 2;                // next entry of the same unit; LEAD: entries of its node
+  int* const cnt = reinterpret_cast<int*>(nxt + (ntab + 1) / 2 % 2 * 2 + a.capi);  // [0] injection, [1] sampling entries, [3] LEAD used, [4 ..] per-warp counts
   volatile int* const aborted = cnt + 2;
   uint32_t* const tab = reinterpret_cast<uint32_t*>(cnt + 4 + C2_THREADS / 32);  // clusters: edge rows of the levels, low parts
   float2* const dmp = reinterpret_cast<float2*>(tab + (BAND ? 0 : 8 * R));
@@ -498,13 +506,23 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
       __syncthreads();
     }
     // a chain of entries per unit, in this order
-    for (int u = tid; u < units; u += C2_THREADS) {
+    for (int u = tid; u < ntab; u += C2_THREADS) {
       ub_[u].z = (int)(NONE << 16 | NONE);
       tl[u] = (uint16_t)NONE;
     }
     if (tid == 0) cnt[3] = 0;
     __syncthreads();
-    if (tid < 32) {
+    if (LEAN) {
+      for (int i = tid; i < ni; i += C2_THREADS) {
+        const uint32_t l = il[i] >> 16;
+        if (i > 0 && il[i - 1] >> 16 == l) continue;
+        int n = 1;
+        while (i + n < ni && il[i + n] >> 16 == l) ++n;
+        il[i] |= LEAD;
+        nxt[i] = (uint16_t)n;
+        cnt[3] = 1;
+      }
+    } else if (tid < 32) {
       for (int b = 0; b < ni; b += 32) {
         const int i = b + tid;
         const bool on = i < ni;
@@ -528,7 +546,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
       }
     }
     __syncthreads();
-    for (int u = tid; u < units; u += C2_THREADS) {
+    for (int u = tid; u < ntab; u += C2_THREADS) {
       const int ch = u / nx4, cu = u - ch * nx4;
       int start, d, row = -1, at[4] = {a.capi, a.capi, a.capi, a.capi};
       march(ch, start, d);
@@ -711,7 +729,16 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
         const uint32_t neff = cur ? sE0 - sU0 / 2u : sE0 + ebytes - (sU0 + lbytes) / 2u;
         for (int un = tid; un < units; un += C2_THREADS) {
           {
-            const int4 A = ldsi4(sA + (uint32_t)un * 16u);
+            int4 A;
+            int cul = 0;  // LEAN: the column
+            if (LEAN) {
+              const int ch = un / nx4, first = ch * N;
+              cul = un - ch * nx4;
+              A = make_int4((first * sx + 4 + 4 * cul) * 4, (z0 + H + first) * px + HX + 4 * cul, 0,
+                            (first < nrow ? F_ON : 0) | (first + N <= nrow ? F_FULL : 0) | first << 8);
+            } else {
+              A = ldsi4(sA + (uint32_t)un * 16u);
+            }
             const int f = A.w;
             if (!(f & F_ON)) continue;
             const int ds = f & F_UP ? -rs : rs, gd = f & F_UP ? -px : px, cd = (f & F_UP ? -nx4 : nx4) * 16;
@@ -727,7 +754,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
                 if (COMP) e = lds2(eoff + x / 2u);
               } else {
                 const int i = cur * 2 * R + (r < 0 ? r + R : r - rpc + R);
-                const uint32_t co = (uint32_t)(4 + 4 * ldsi(sB + (uint32_t)un * 16u + 12u));
+                const uint32_t co = (uint32_t)(4 + 4 * (LEAN ? cul : ldsi(sB + (uint32_t)un * 16u + 12u)));
                 u = ldc4(tab[i] + co * 4u);
                 if (COMP) e = ldc2(tab[4 * R + i] + co * 2u);
               }
@@ -780,6 +807,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
             for (int b = 0; b < N / BL; ++b) {
 #pragma unroll
               for (int jj = 0; jj < BL; ++jj) {
+                if (LEAN && start + jj >= rpc) break;  // the last chunk's rows
                 // the row R beyond this one completes the queue (bands: a row of the next chunk at most)
                 if (BAND) {
                   u[jj + 2 * R] = lds4(ha);
@@ -836,7 +864,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
             }
           }
           // entries at this unit's points, added to the values just stored
-          const uint32_t ent = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
+          const uint32_t ent = LEAN ? NONE << 16 | NONE : (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
           if (ent != (NONE << 16 | NONE)) {
             const int f = ldsi(sA + (uint32_t)un * 16u + 12u), start = f >> 8, d = f & F_UP ? -1 : 1;
             const int cu = ldsi(sB + (uint32_t)un * 16u + 12u);
@@ -967,7 +995,7 @@ int c2_cap(int n) { return (std::max(n, 1) + 3) / 4 * 4; }
 
 // shared memory of a band of rpc rows (chunks of N)
 size_t c2_bytes(int rpc, int N, int sx, int nx4, int R, int mode, bool band, bool c2s, int sw, int capi, int caps) {
-  const size_t units = (size_t)(rpc / N) * nx4;
+  const size_t units = band || c2s ? (size_t)(rpc / N) * nx4 : 0;  // with entries in the tables (lean: none)
   size_t b = (size_t)(2 * rpc + (band ? 0 : 1)) * sx * 4;   // both levels, zero row
   if (mode == C2_COMP) b += (size_t)(2 * rpc + (band ? 3 * R : 0)) * sx * 2;  // low parts of both levels (bf16)
   if (c2s) b += (size_t)rpc * nx4 * 16;                     // c2
@@ -980,7 +1008,9 @@ size_t c2_bytes(int rpc, int N, int sx, int nx4, int R, int mode, bool band, boo
 }
 
 // Whether a shot of this grid fits one cluster of C CTAs, for the acceptance
-// of the compensated form; the kernel itself needs no more than this.
+// of the compensated form: an upper bound of what a lean cluster of these CTAs
+// needs (c2_bytes without c2: at least 32 rpc + 32 R + 2 cap - 40 bytes less), so
+// that every grid accepted has a plan.
 bool c2_accepts(const Layout& L, int R, int C, bool comp, int cap) {
   const int nx4 = (L.nx + 3) / 4, sx = 4 * nx4 + 8;
   const int rpc = (L.nz + C - 1) / C;
@@ -997,8 +1027,8 @@ struct C2Plan {
   double est = 0;
 };
 
-// rows per unit: bands (few units: short marches), clusters
-constexpr int C2_NB = 8, C2_NS = 4, C2_NC = 2, C2_N1 = 1;
+// rows per unit: bands (few units: short marches), clusters, lean clusters
+constexpr int C2_NB = 8, C2_NS = 4, C2_NC = 2, C2_N1 = 1, C2_NL = 4;
 
 // Estimated us of a step of a band of rpc rows, from measurements on GB300 (a
 // pass marches w warps of units; every unit fills its queue with 2R rows).
@@ -1007,8 +1037,8 @@ constexpr int C2_NB = 8, C2_NS = 4, C2_NC = 2, C2_N1 = 1;
 // 201 2.1 / 2.1, 401 x 401 4.5 / 4.3, 300 x 70 x 40 3.4 / 3.3, compensated 201 x
 // 201 2.95 / 2.9.  Below them an exchange through L2 (bands) or a march's
 // latency decides.
-double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band) {
-  const int units = rpc / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
+double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band, int c2s) {
+  const int units = (rpc + N - 1) / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
   const double w = std::min(16, (units + 31) / 32);
   if (band) {
     const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : (mode == C2_DAMP ? 0.026 : 0.0185);
@@ -1019,23 +1049,21 @@ double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band) {
   return (N == 1 ? 1.25 : 1.4) + passes * w * (N * row + 2 * R * fill);
 }
 
-C2Plan c2_try(const Layout& L, int R, int mode, int sw, int nshots, int C, int N, int groups, bool band, int capi, int caps) {
+// c2s 0: c2 in global memory (bands; lean clusters)
+C2Plan c2_try(const Layout& L, int R, int mode, int sw, int nshots, int C, int N, int groups, bool band, int c2s, int capi,
+              int caps) {
   C2Plan p;
   const int nx4 = (L.nx + 3) / 4, sx = 4 * nx4 + 8;
   if (nx4 > C2_MAXCOL || groups < 1) return p;
+  const int rows = (L.nz + C - 1) / C;
   // bands: at least two chunks, so that the rows beyond a chunk are in the band
-  const int rpc = std::max(((L.nz + C - 1) / C + N - 1) / N, band ? 2 : 1) * N;
+  const int rpc = !band && !c2s ? rows : std::max((rows + N - 1) / N, band ? 2 : 1) * N;
   if ((L.nz + rpc - 1) / rpc != C) return p;  // no empty bands
   if ((size_t)rpc * sx > 65535) return p;  // the lists keep band indices in 16 bits
-  int c2s = 1;
-  size_t sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, true, sw, capi, caps);
-  if (sm > C2_SMEM && band) {
-    c2s = 0;
-    sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, false, sw, capi, caps);
-  }
+  const size_t sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, c2s, sw, capi, caps);
   if (sm > C2_SMEM) return p;
   p.C = C; p.rpc = rpc; p.N = N; p.groups = std::min(groups, nshots); p.c2s = c2s; p.band = band; p.smem = sm;
-  p.est = (double)((nshots + p.groups - 1) / p.groups) * c2_step_cost(rpc, N, nx4, R, mode, band);
+  p.est = (double)((nshots + p.groups - 1) / p.groups) * c2_step_cost(rpc, N, nx4, R, mode, band, c2s);
   return p;
 }
 
@@ -1055,19 +1083,24 @@ C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, 
   const int sms = c2_sms();
   for (int C = 1; C <= sms; ++C)
     for (int N : {C2_NB, C2_NS}) {
-      const C2Plan p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, capi, caps);
+      C2Plan p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 1, capi, caps);
+      if (!p.C) p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 0, capi, caps);
       if (p.C && (!best.C || p.est < best.est)) best = p;
     }
   return best;
 }
 
-// clusters of C CTAs with `smem` bytes each that fit on the current device at once (cached)
-template <int R, int MODE, int N>
+// clusters of C CTAs with `smem` bytes each that fit on the current device at
+// once (cached); without a device, a guess for planning
+template <int R, int MODE, int N, bool C2S>
 int c2_max_clusters(int C, size_t smem) {
   static std::mutex m;
   static std::vector<std::pair<long long, int>> cache;
   int dev = 0;
-  cudaGetDevice(&dev);
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return std::max(1, C2_MAXBANDS / 2 / C);
+  }
   const long long key = ((long long)dev << 40) | ((long long)C << 32) | (long long)smem;
   {
     std::lock_guard<std::mutex> lk(m);
@@ -1086,7 +1119,8 @@ int c2_max_clusters(int C, size_t smem) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, sweep2d_shots<R, MODE, false, N, true>, &cfg) != cudaSuccess) {
+  if (smem_limit_once<sweep2d_shots<R, MODE, false, N, C2S>>((int)C2_SMEM, true) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, sweep2d_shots<R, MODE, false, N, C2S>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     n = 0;
   }
@@ -1098,14 +1132,19 @@ int c2_max_clusters(int C, size_t smem) {
 template <int R, int MODE>
 C2Plan c2_choose(const Layout& L, int sw, int nshots, int capi, int caps) {
   C2Plan best = c2_bands(L, R, MODE, sw, nshots, capi, caps);
-  for (int C = 1; C <= C2_MAXC; ++C)
-    for (int N : {C2_NC, C2_N1}) {
-      C2Plan p = c2_try(L, R, MODE, sw, nshots, C, N, nshots, false, capi, caps);
-      if (!p.C) continue;
-      const int ncl = N == C2_N1 ? c2_max_clusters<R, MODE, C2_N1>(C, p.smem) : c2_max_clusters<R, MODE, C2_NC>(C, p.smem);
-      p = c2_try(L, R, MODE, sw, nshots, C, N, ncl, false, capi, caps);
-      if (p.C && (!best.C || p.est < best.est)) best = p;
-    }
+  auto cluster = [&](int C, int N, int c2s, auto at_once) {
+    C2Plan p = c2_try(L, R, MODE, sw, nshots, C, N, nshots, false, c2s, capi, caps);
+    if (!p.C) return;
+    p = c2_try(L, R, MODE, sw, nshots, C, N, at_once(C, p.smem), false, c2s, capi, caps);
+    if (p.C && (!best.C || p.est < best.est)) best = p;
+  };
+  for (int C = 1; C <= C2_MAXC; ++C) {
+    cluster(C, C2_NC, 1, c2_max_clusters<R, MODE, C2_NC, true>);
+    cluster(C, C2_N1, 1, c2_max_clusters<R, MODE, C2_N1, true>);
+  }
+  if constexpr (MODE != C2_DAMP)
+    if (!best.C)
+      for (int C = 1; C <= C2_MAXC; ++C) cluster(C, C2_NL, 0, c2_max_clusters<R, MODE, C2_NL, false>);
   return best;
 }
 
@@ -1134,11 +1173,17 @@ cudaError_t c2_run(const C2Args& a, const C2Plan& pl, cudaStream_t s) {
   return l != cudaSuccess ? l : cudaGetLastError();
 }
 
+C2Plan c2_plan(const Layout& L, const Weights& W, int mode, int nshots, int ninj, int nsamp) {
+  const int capi = c2_cap(ninj), caps = c2_cap(nsamp);
+#define TP_C2(RR) (mode == C2_COMP ? c2_choose<RR, C2_COMP>(L, W.sw, nshots, capi, caps)                       \
+                                   : (mode == C2_DAMP ? c2_choose<RR, C2_DAMP>(L, W.sw, nshots, capi, caps)    \
+                                                      : c2_choose<RR, C2_LEVELS>(L, W.sw, nshots, capi, caps)))
+  return W.R == 4 ? TP_C2(4) : TP_C2(2);
+#undef TP_C2
+}
+
 template <int R, int MODE>
 cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
-  cudaError_t e = smem_limit_once<sweep2d_shots<R, MODE, false, C2_NC, true>>((int)C2_SMEM, true);  // before the occupancy query
-  if (e == cudaSuccess) e = smem_limit_once<sweep2d_shots<R, MODE, false, C2_N1, true>>((int)C2_SMEM, true);
-  if (e != cudaSuccess) return e;
   C2Args a = a0;
   a.capi = c2_cap(a.ninj);
   a.caps = c2_cap(a.nsamp);
@@ -1148,6 +1193,8 @@ cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
   a.rpc = pl.rpc;
   a.nx4 = (a.L.nx + 3) / 4;
   a.sx = 4 * a.nx4 + 8;
+  if constexpr (MODE != C2_DAMP)
+    if (!pl.band && !pl.c2s) return c2_run<R, MODE, false, C2_NL, false>(a, pl, s);
   if (!pl.band) return pl.N == C2_N1 ? c2_run<R, MODE, false, C2_N1, true>(a, pl, s) : c2_run<R, MODE, false, C2_NC, true>(a, pl, s);
   if (pl.N == C2_NS)
     return pl.c2s ? c2_run<R, MODE, true, C2_NS, true>(a, pl, s) : c2_run<R, MODE, true, C2_NS, false>(a, pl, s);
@@ -1171,6 +1218,12 @@ bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int
   if (L.ndim != 2 || nsrc > C2_MAXLIST || nrec > C2_MAXLIST) return false;
   const int cap = c2_cap(std::max(nsrc, nrec));
   return c2_bands(L, W.R, W.sw > 0 ? C2_DAMP : C2_LEVELS, W.sw, nshots, cap, cap).C > 0;
+}
+
+void plan2d(const Layout& L, const Weights& W, bool comp, int nshots, int ninj, int nsamp, int plan[6]) {
+  const C2Plan p = c2_plan(L, W, comp ? C2_COMP : (W.sw > 0 ? C2_DAMP : C2_LEVELS), nshots, ninj, nsamp);
+  const int v[6] = {p.C ? (p.band ? 1 : 2) : 0, p.C, p.rpc, p.N, p.groups, p.c2s};
+  std::copy(v, v + 6, plan);
 }
 
 size_t edge2d_bytes(const Layout& L, const Weights& W) {

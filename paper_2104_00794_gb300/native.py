@@ -88,12 +88,13 @@ def lib():
         L.tp_profile_end.argtypes = [ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int64)]
         L.tp_set_wait_limit.argtypes = [ctypes.c_int64]
         L.tp_form_supported.argtypes = [G, E]
+        L.tp_sweep2d_plan.argtypes = [G, E, i32, ctypes.POINTER(i32)]
         L.tp_kernel_name.argtypes = [i32]
         L.tp_kernel_name.restype = ctypes.c_char_p
         for f in ("tp_forward", "tp_adjoint", "tp_gradient_probed", "tp_gradient_full", "tp_probes",
                   "tp_workspace_status", "tp_profile_begin", "tp_profile_end", "tp_misfit_noalloc",
                   "tp_probed_forward", "tp_probed_backward", "tp_qr_probes", "tp_probed_image", "tp_residual",
-                  "tp_set_wait_limit", "tp_form_supported"):
+                  "tp_set_wait_limit", "tp_form_supported", "tp_sweep2d_plan"):
             getattr(L, f).restype = ctypes.c_int
         _lib = L
         return L
@@ -199,6 +200,14 @@ def tp_form_supported(grid, geom) -> bool:
     """Whether the library can run `grid` (its time form in particular) for
     batches with geom's counts (no device work)."""
     return lib().tp_form_supported(ctypes.byref(grid), ctypes.byref(geom)) == TP_OK
+
+
+def tp_sweep2d_plan(grid, geom, adjoint: bool = False) -> tuple:
+    """How batches on `grid` are stepped: (0 a launch per step, 1 bands of a cooperative grid, 2 a
+    cluster per shot; CTAs per shot, rows per CTA, rows per march, shots at once, c2 in shared memory)."""
+    plan = (ctypes.c_int * 6)()
+    _check(lib().tp_sweep2d_plan(ctypes.byref(grid), ctypes.byref(geom), int(adjoint), plan))
+    return tuple(plan)
 
 
 def tp_set_wait_limit(cycles: int):
