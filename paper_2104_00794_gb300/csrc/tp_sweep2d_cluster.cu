@@ -77,7 +77,7 @@ constexpr int C2_MAXC = 16;      // cluster size limit (non-portable above 8)
 constexpr int C2_MAXBANDS = 152; // CTAs of a cooperative launch
 constexpr size_t C2_SMEM = 227 * 1024;
 
-enum C2Mode { C2_LEVELS = 0, C2_COMP = 1, C2_DAMP = 2 };
+enum C2Mode { C2_LEVELS = 0, C2_COMP = 1, C2_DAMP = 2 };  // (index the tables of c2_step_cost)
 struct C2Args {
   Layout L;
   Weights W;
@@ -1027,26 +1027,63 @@ struct C2Plan {
   double est = 0;
 };
 
-// rows per unit: bands (few units: short marches), clusters, lean clusters
-constexpr int C2_NB = 8, C2_NS = 4, C2_NC = 2, C2_N1 = 1, C2_NL = 4;
+// rows that the marches of a column read from neighbouring CTAs
+int c2_remote(int rpc, int N, int R) {
+  int n = 0;
+  for (int a = 0; a < rpc; a += N) n += std::max(0, R - a) + std::max(0, std::min(a + N, rpc) + R - rpc);
+  return n;
+}
 
-// Estimated us of a step of a band of rpc rows, from measurements on GB300 (a
-// pass marches w warps of units; every unit fills its queue with 2R rows).
-// Measured / estimated: bands, levels, 601 x 201 x 16 shots 3.9 / 4.2, 801 x 301
-// x 8 3.9 / 4.0, compensated 8.2 / 9.3 and 8.0 / 9.3; clusters, levels, 201 x
-// 201 2.1 / 2.1, 401 x 401 4.5 / 4.3, 300 x 70 x 40 3.4 / 3.3, compensated 201 x
-// 201 2.95 / 2.9.  Below them an exchange through L2 (bands) or a march's
-// latency decides.
+// Estimated us of a step in which every CTA has rpc rows, marched N at a time
+// (rows of nx4 columns, units of 32 per warp): a sum of the rows marched, the
+// 2R queue rows that every march fills, the passes of the CTA's threads, a
+// march's latency and, in clusters, the rows read from a neighbour's shared
+// memory.  The coefficients are a least-squares fit (relative, non-negative) to
+// 9686 measured splits of 260 random grids (8 to 2048 x 16 to 420, 1 to 40 shots,
+// both orders, all modes); mean error 3 to 8 %.  The split with the least
+// estimate, with the bands' split from c2_band_rank, takes on average 2.8 %
+// longer than the best of the measured ones (at most 26 %).  Costs without the
+// remote rows, and without clusters of 4 rows a march: 6.3 % (93 %; 1500 x 60
+// 5.0 us a step instead of 2.8, 601 x 201 4.7 instead of 3.5).
 double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band, int c2s) {
   const int units = (rpc + N - 1) / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
-  const double w = std::min(16, (units + 31) / 32);
+  const double u = units / 32.0, order8 = R == 4;
   if (band) {
-    const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : (mode == C2_DAMP ? 0.026 : 0.0185);
-    const double floor = R == 4 ? 3.6 : (N == 8 ? 1.9 : 1.5) * (mode == C2_COMP ? 1.45 : 1.0);
-    return std::max(floor, (mode == C2_COMP ? 1.9 : 1.6) + passes * N * row * w) + 0.03 * passes * w;
+    // [mode]: constant, order 8, warps, latency by N, columns, passes, rows (N = 8), rows (c2 in global memory), rows (order 8)
+    static const double K[3][9] = {{1.176, 1.122, 0., 0., 0.306, 0.660, 0.0061, 0.0058, 0.0005},
+                                   {0.033, 0.869, 0.0472, 0.170, 0.336, 1.273, 0.0096, 0.0051, 0.0144},
+                                   {0., 0.922, 0.0395, 0.411, 0.108, 1.175, 0.0075, 0.0058, 0.0064}};
+    const double* k = K[mode];
+    return k[0] + k[1] * order8 + k[2] * u + k[3] * N + k[4] * nx4 / 100 + k[5] * passes +
+           u * N * (k[6] * (N == 8) + k[7] * !c2s + k[8] * order8);
   }
-  const double row = mode == C2_COMP ? 0.05 : (mode == C2_DAMP ? 0.024 : 0.02), fill = mode == C2_COMP ? 0.004 : 0.0025;
-  return (N == 1 ? 1.25 : 1.4) + passes * w * (N * row + 2 * R * fill);
+  if (!c2s) {  // lean: constant, order 8, rows filled, passes, remote rows
+    static const double K[2][5] = {{1.487, 0.139, 0.0053, 0.907, 0.0037}, {1.362, 0.611, 0.0161, 1.330, 0.}};
+    const double* k = K[mode];
+    return k[0] + k[1] * order8 + k[2] * u * 2 * R + k[3] * passes + k[4] * c2_remote(rpc, N, R) * nx4 / 1000;
+  }
+  // clusters, [mode]: constant, order 8, rows marched, rows filled, remote rows, latency by N, passes
+  static const double K[3][7] = {{0.964, 0.259, 0.0103, 0.0023, 0.137, 0.133, 0.325},
+                                 {0.899, 0.428, 0.0227, 0.0048, 0.224, 0.241, 0.346},
+                                 {0.912, 0.263, 0.0206, 0.0006, 0.128, 0.348, 0.480}};
+  const double* k = K[mode];
+  return k[0] + k[1] * order8 + k[2] * u * N + k[3] * u * 2 * R + k[4] * c2_remote(rpc, N, R) * nx4 / 1000 + k[5] * N +
+         k[6] * passes;
+}
+
+// Rank of a split into bands among splits into bands: a step's time with the
+// floor that the exchange sets (3.6 us at order 8).  Near the floor the phases of
+// the exchange decide, by up to 25 % and not smoothly; the fit above has no
+// floor and picked shorter marches there (601 x 201 x 16 shots 4.2 us instead of
+// 3.9, 397 x 401 x 4 3.8 instead of 3.1), but it tells the splits at the floor
+// apart (601 x 201: 26 bands of 8 rows 3.5 us, 13 of 16 4.1): a fifth of it counts.
+// (With a layer the marches are longer and the fit alone ranks better.)
+double c2_band_rank(int rpc, int N, int nx4, int R, int mode) {
+  const int units = rpc / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
+  const double w = std::min(16, (units + 31) / 32);
+  const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : 0.0185;
+  const double floor = R == 4 ? 3.6 : (N == 8 ? 1.9 : 1.5) * (mode == C2_COMP ? 1.45 : 1.0);
+  return std::max(floor, (mode == C2_COMP ? 1.9 : 1.6) + passes * N * row * w) + 0.03 * passes * w;
 }
 
 // c2s 0: c2 in global memory (bands; lean clusters)
@@ -1077,15 +1114,22 @@ int c2_sms() {
   return std::min(sms, C2_MAXBANDS);
 }
 
-// The best split into bands of one cooperative grid (est = 0: none fits)
+// The best split into bands of one cooperative grid (C = 0: none fits)
 C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, int caps) {
   C2Plan best;
+  double least = 0;
   const int sms = c2_sms();
   for (int C = 1; C <= sms; ++C)
-    for (int N : {C2_NB, C2_NS}) {
+    for (int N : {8, 4}) {
       C2Plan p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 1, capi, caps);
       if (!p.C) p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 0, capi, caps);
-      if (p.C && (!best.C || p.est < best.est)) best = p;
+      if (!p.C) continue;
+      const double rounds = (nshots + p.groups - 1) / p.groups;
+      const double rank =
+          mode == C2_DAMP ? p.est : rounds * c2_band_rank(p.rpc, N, (L.nx + 3) / 4, R, mode) + 0.2 * p.est;
+      if (best.C && rank >= least) continue;
+      best = p;
+      least = rank;
     }
   return best;
 }
@@ -1139,12 +1183,11 @@ C2Plan c2_choose(const Layout& L, int sw, int nshots, int capi, int caps) {
     if (p.C && (!best.C || p.est < best.est)) best = p;
   };
   for (int C = 1; C <= C2_MAXC; ++C) {
-    cluster(C, C2_NC, 1, c2_max_clusters<R, MODE, C2_NC, true>);
-    cluster(C, C2_N1, 1, c2_max_clusters<R, MODE, C2_N1, true>);
+    cluster(C, 4, 1, c2_max_clusters<R, MODE, 4, true>);
+    cluster(C, 2, 1, c2_max_clusters<R, MODE, 2, true>);
+    cluster(C, 1, 1, c2_max_clusters<R, MODE, 1, true>);
+    if constexpr (MODE != C2_DAMP) cluster(C, 4, 0, c2_max_clusters<R, MODE, 4, false>);
   }
-  if constexpr (MODE != C2_DAMP)
-    if (!best.C)
-      for (int C = 1; C <= C2_MAXC; ++C) cluster(C, C2_NL, 0, c2_max_clusters<R, MODE, C2_NL, false>);
   return best;
 }
 
@@ -1193,12 +1236,15 @@ cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
   a.rpc = pl.rpc;
   a.nx4 = (a.L.nx + 3) / 4;
   a.sx = 4 * a.nx4 + 8;
+  if (pl.band) {
+    if (pl.N == 4) return pl.c2s ? c2_run<R, MODE, true, 4, true>(a, pl, s) : c2_run<R, MODE, true, 4, false>(a, pl, s);
+    return pl.c2s ? c2_run<R, MODE, true, 8, true>(a, pl, s) : c2_run<R, MODE, true, 8, false>(a, pl, s);
+  }
   if constexpr (MODE != C2_DAMP)
-    if (!pl.band && !pl.c2s) return c2_run<R, MODE, false, C2_NL, false>(a, pl, s);
-  if (!pl.band) return pl.N == C2_N1 ? c2_run<R, MODE, false, C2_N1, true>(a, pl, s) : c2_run<R, MODE, false, C2_NC, true>(a, pl, s);
-  if (pl.N == C2_NS)
-    return pl.c2s ? c2_run<R, MODE, true, C2_NS, true>(a, pl, s) : c2_run<R, MODE, true, C2_NS, false>(a, pl, s);
-  return pl.c2s ? c2_run<R, MODE, true, C2_NB, true>(a, pl, s) : c2_run<R, MODE, true, C2_NB, false>(a, pl, s);
+    if (!pl.c2s) return c2_run<R, MODE, false, 4, false>(a, pl, s);
+  return pl.N == 4   ? c2_run<R, MODE, false, 4, true>(a, pl, s)
+         : pl.N == 2 ? c2_run<R, MODE, false, 2, true>(a, pl, s)
+                     : c2_run<R, MODE, false, 1, true>(a, pl, s);
 }
 
 }  // namespace

@@ -88,3 +88,32 @@ def test_wide_grids_run_the_default_form(cuda_lib, nx, nz, nshots, order, nrec):
     p.status(native.OP_GRADIENT_PROBED)
     ref, _ = oracle.batch_gradient_probed(w, w.vel0, dobs, kind="rademacher", r=4, seed=w.seed)
     assert rel_l2(host(gp), ref) <= 1e-4
+
+
+@pytest.mark.gpu
+def test_less_work_does_not_take_longer(cuda_lib):
+    """A split is taken by an estimate; with a wrong one a sixth of the rows took
+    as long as all of them (1500 x 60 against 1500 x 400), and one shot longer
+    than sixteen (601 x 201)."""
+    import dataclasses
+
+    import torch
+
+    from parity_util import problem, to_dev
+
+    def ms(nx, nz, nshots):
+        w = wl.small_2d(nx=nx, nz=nz, nt=200, order=8, nshots=nshots)
+        w = dataclasses.replace(w, rec=w.rec[:, ::2].copy())  # at most 1024: more are stepped a launch at a time
+        p, v, q = problem(w), to_dev(w.vel0), to_dev(w.wavelet)
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            p.forward(v, q)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    assert ms(1500, 60, 1) <= 0.8 * ms(1500, 400, 1)
+    assert ms(601, 201, 1) <= ms(601, 201, 16)
