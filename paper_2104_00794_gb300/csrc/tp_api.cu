@@ -253,7 +253,7 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
     P->pt_bytes = cur - P->o_pt;
     for (int i = 0; i < 2; ++i) {
       P->o_pt_base[i] = take(cur, segs * sizeof(int));
-      P->o_pt_ent[i] = take(cur, (size_t)ns * (i ? P->nrec : P->nsrc) * sizeof(int));
+      P->o_pt_ent[i] = take(cur, (size_t)4 * ns * (i ? P->nrec : P->nsrc) * sizeof(int));  // ent, num, work
     }
   }
   P->c2_bytes = fb + (P->L.ndim == 2 ? (size_t)8 * P->L.plane * sizeof(float) : 0);  // + rows that a 2-D band's last chunk reads
@@ -372,6 +372,8 @@ PointTiles point_tiles(const Ctx& c, int set) {
   t.count = reinterpret_cast<int*>(b + segs * 16 + words * 4);
   t.base = c.at<int>(P.o_pt_base[set]);
   t.ent = c.at<int>(P.o_pt_ent[set]);
+  t.num = t.ent + (size_t)P.nshots * (set ? P.nrec : P.nsrc);
+  t.work = t.num + (size_t)P.nshots * (set ? P.nrec : P.nsrc);
   return t;
 }
 
@@ -391,9 +393,9 @@ tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float*
   if (P.L.ndim == 3) {  // the sweeps inject
     TRY(cudaMemsetAsync(c.at<char>(P.o_pt), 0, P.pt_bytes, c.st));
     TRY(launch_point_tiles(P.L, c.at<long long>(P.o_soff), P.nsrc, P.nshots, point_tiles(c, 0),
-                           c.at<unsigned char>(P.o_salone), c.at<int>(P.o_sshared), c.at<int>(P.o_sn), c.st));
+                           c.at<unsigned char>(P.o_salone), c.at<int>(P.o_sshared), c.st));
     TRY(launch_point_tiles(P.L, c.at<long long>(P.o_roff), P.nrec, P.nshots, point_tiles(c, 1),
-                           c.at<unsigned char>(P.o_ralone), c.at<int>(P.o_rshared), c.at<int>(P.o_rn), c.st));
+                           c.at<unsigned char>(P.o_ralone), c.at<int>(P.o_rshared), c.st));
   } else {
     // injection groups; the wavefield block (at least one field per shot, zeroed
     // by every operation after the set-up) serves as the count scratch

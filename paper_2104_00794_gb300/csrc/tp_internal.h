@@ -92,8 +92,9 @@ struct FieldRef {
 // 3-D: the entries of a point set by grid row, for the sweep that injects them
 // into the points it forms.  A segment is 64 consecutive nodes of a row
 // (segment (z * ny + y) * ntx + x / 64 of a shot, ntx = ceil(nx / 64)); entry e
-// of segment s (in node order) is ent[shot][base[s] + e]: the index of the only
-// entry at that node, or -1 where several share it (they are in `shared`).
+// of segment s (in node order) is slot base[s] + e of its shot: ent holds the
+// index of the only entry at that node, or -2 - p where several share it: those
+// num[slot] entries are, in index order, inj_shared[shot][p ..].
 // tile: a bit per plane for every 64 x 16 column of the grid.
 constexpr int PT_X = 64, PT_Y = 16;
 struct PointTiles {
@@ -102,7 +103,9 @@ struct PointTiles {
   unsigned long long* dup;    // [shot][segments]: nodes with several
   int* base;                  // [shot][segments]
   int* ent;                   // [shot][entries]
-  int* count;                 // [shot][2] scratch: entries placed, entries that share a node
+  int* num;                   // [shot][entries]
+  int* work;                  // [shot][2][entries] scratch
+  int* count;                 // [shot][2] scratch: slots placed, entries that share a node
 };
 __host__ __device__ inline int pt_tx(const Layout& L) { return (L.nx + PT_X - 1) / PT_X; }
 __host__ __device__ inline int pt_words(const Layout& L) { return (L.nz + 31) / 32; }
@@ -115,7 +118,8 @@ inline long long pt_segs(const Layout& L) { return (long long)L.nz * L.ny * pt_t
 //   srcacc (optional): acc[s][j] += sampled value * acc_val[s][t_a][j]
 // Injection is deterministic: entries alone at their node (inj_alone[s][k])
 // are added by their own thread, the others (inj_shared[s][0 .. inj_nshared[s]),
-// in index order) by one thread per shot, one after the other.
+// in index order) by one thread per shot, one after the other.  In 3-D the sweep
+// injects, by node (PointTiles).
 struct PointArgs {
   int nshots;
   const float* field_samp; long long samp_ss;
@@ -240,9 +244,9 @@ cudaError_t launch_point(const PointArgs& a, cudaStream_t s);
 // padded offsets; cnt_scratch: nshots * field ints of scratch
 cudaError_t launch_point_groups(const long long* off, int per_shot, int nshots, long long field, int* cnt_scratch,
                                 unsigned char* alone, int* shared, int* nshared, cudaStream_t s);
-// 3-D: the same set as `tiles` (tile, mask, dup and count zero on entry), shared and nshared; flags: n bytes of scratch
+// 3-D: the set as `tiles` (tile, mask, dup and count zero on entry) and shared; flags: n bytes of scratch
 cudaError_t launch_point_tiles(const Layout& L, const long long* off, int per_shot, int nshots, const PointTiles& tiles,
-                               unsigned char* flags, int* shared, int* nshared, cudaStream_t s);
+                               unsigned char* flags, int* shared, cudaStream_t s);
 
 cudaError_t launch_probes(int kind, int nt, int r, uint64_t seed, int shot0, int nshots,
                           const float* Z_user, float* Q, cudaStream_t s);

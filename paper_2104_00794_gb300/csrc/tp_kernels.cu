@@ -152,6 +152,15 @@ __device__ __forceinline__ PtPos pt_pos(const Layout& L, long long o, int* tile_
   return PtPos{(z * L.ny + y) * ntx + x / PT_X, x % PT_X};
 }
 
+// the slot of entry k of shot s (entry at offset o) in ent, and its segment
+__device__ __forceinline__ long long pt_slot(const Layout& L, const PointTiles& t, long long segs, long long s,
+                                             int per_shot, long long o, long long* seg, unsigned long long* bit) {
+  const PtPos p = pt_pos(L, o, nullptr, nullptr);
+  *seg = s * segs + p.seg;
+  *bit = 1ULL << p.bit;
+  return s * per_shot + t.base[*seg] + __popcll(t.mask[*seg] & (*bit - 1));
+}
+
 // step 0: masks, and flags[k] = 1 for the first entry of a segment; step 1:
 // these place their segment; step 2: every entry writes its slot
 __global__ void point_tiles_kernel(Layout L, const long long* __restrict__ off, long long n, int per_shot,
@@ -162,47 +171,69 @@ __global__ void point_tiles_kernel(Layout L, const long long* __restrict__ off, 
       flags[k] = 0;
       continue;
     }
+    if (step == 2) {
+      long long seg;
+      unsigned long long bit;
+      const long long slot = pt_slot(L, t, segs, s, per_shot, o, &seg, &bit);
+      const bool several = (t.dup[seg] & bit) != 0;
+      t.ent[slot] = several ? -1 : (int)(k % per_shot);
+      t.num[slot] = 0;
+      flags[k] = several ? 2 : 0;
+      if (several) atomicAdd(t.count + 2 * s + 1, 1);
+      continue;
+    }
     int tw = 0, tb = 0;
     const PtPos p = pt_pos(L, o, &tw, &tb);
     const long long seg = s * segs + p.seg;
-    const unsigned long long bit = 1ULL << p.bit;
     if (step == 0) {
-      const unsigned long long had = atomicOr(t.mask + seg, bit);
+      const unsigned long long bit = 1ULL << p.bit, had = atomicOr(t.mask + seg, bit);
       if (had & bit) atomicOr(t.dup + seg, bit);
       flags[k] = had == 0 ? 1 : 0;
       atomicOr(t.tile + s * tile_words + tw, 1u << tb);
-    } else if (step == 1) {
-      if (flags[k]) t.base[seg] = atomicAdd(t.count + 2 * s, __popcll(t.mask[seg]));
-    } else {
-      const bool several = (t.dup[seg] & bit) != 0;
-      t.ent[s * per_shot + t.base[seg] + __popcll(t.mask[seg] & (bit - 1))] = several ? -1 : (int)(k % per_shot);
-      flags[k] = several ? 2 : 0;
-      if (several) atomicAdd(t.count + 2 * s + 1, 1);
+    } else if (flags[k]) {
+      t.base[seg] = atomicAdd(t.count + 2 * s, __popcll(t.mask[seg]));
     }
   }
 }
 
-// one block per shot: the entries that share a node (flags[k] = 2), in index order
-__global__ void __launch_bounds__(256) point_shared_kernel(const unsigned char* __restrict__ flags, int per_shot,
-                                                           const int* __restrict__ count, int* shared, int* nshared) {
-  __shared__ int warp_cnt[8];
+// One block per shot: the entries that share a node (flags[k] = 2), listed by
+// node and in index order at a node: entries of a slot are counted, placed, and
+// ranked among those of their slot.
+__global__ void __launch_bounds__(1024) point_shared_kernel(Layout L, const long long* __restrict__ off, int per_shot,
+                                                            long long segs, PointTiles t,
+                                                            const unsigned char* __restrict__ flags, int* list) {
+  __shared__ int total;
   const int s = blockIdx.x, tid = threadIdx.x;
-  int base = 0;
-  if (count[2 * s + 1] > 0)
-    for (int b = 0; b < per_shot; b += 256) {
-      const bool dup = b + tid < per_shot && flags[(long long)s * per_shot + b + tid] == 2;
-      const unsigned m = __ballot_sync(0xffffffffu, dup);
-      if ((tid & 31) == 0) warp_cnt[tid >> 5] = __popc(m);
-      __syncthreads();
-      int before = base;
-      for (int w = 0; w < 8; ++w) {
-        if (w < (tid >> 5)) before += warp_cnt[w];
-        base += warp_cnt[w];
+  if (t.count[2 * s + 1] == 0) return;
+  if (tid == 0) total = 0;
+  off += (long long)s * per_shot;
+  flags += (long long)s * per_shot;
+  list += (long long)s * per_shot;
+  int* const arrived = t.work + 2LL * s * per_shot;  // entries of its slot before this one (any order)
+  int* const placed = arrived + per_shot;
+  for (int step = 0; step < 4; ++step) {
+    __syncthreads();
+    for (int k = tid; k < per_shot; k += 1024) {
+      if (flags[k] != 2) continue;
+      long long seg;
+      unsigned long long bit;
+      const long long slot = pt_slot(L, t, segs, s, per_shot, off[k], &seg, &bit);
+      if (step == 0) {
+        arrived[k] = atomicAdd(t.num + slot, 1);
+      } else if (step == 1) {
+        if (arrived[k] == 0) t.ent[slot] = -2 - atomicAdd(&total, t.num[slot]);
+      } else {
+        const int first = -2 - t.ent[slot];
+        if (step == 2) {
+          placed[first + arrived[k]] = k;
+        } else {
+          int rank = 0;
+          for (int i = 0; i < t.num[slot]; ++i) rank += placed[first + i] < k;
+          list[first + rank] = k;
+        }
       }
-      if (dup) shared[(long long)s * per_shot + before + __popc(m & ((1u << (tid & 31)) - 1u))] = b + tid;
-      __syncthreads();
     }
-  if (tid == 0) nshared[s] = base;
+  }
 }
 
 // SplitMix64 (Steele, Lea & Flood 2014): the n-th output of a generator whose
@@ -462,12 +493,12 @@ cudaError_t launch_point_groups(const long long* off, int per_shot, int nshots, 
 }
 
 cudaError_t launch_point_tiles(const Layout& L, const long long* off, int per_shot, int nshots, const PointTiles& t,
-                               unsigned char* flags, int* shared, int* nshared, cudaStream_t s) {
+                               unsigned char* flags, int* shared, cudaStream_t s) {
   prof_before(5, s);
   const long long n = (long long)nshots * per_shot, tile_words = pt_tiles(L) * pt_words(L);
   for (int step = 0; step < 3; ++step)
     point_tiles_kernel<<<grid_for(n, 256), 256, 0, s>>>(L, off, n, per_shot, pt_segs(L), tile_words, t, flags, step);
-  point_shared_kernel<<<nshots, 256, 0, s>>>(flags, per_shot, t.count, shared, nshared);
+  point_shared_kernel<<<nshots, 1024, 0, s>>>(L, off, per_shot, pt_segs(L), t, flags, shared);
   prof_after(5, s);
   return cudaGetLastError();
 }

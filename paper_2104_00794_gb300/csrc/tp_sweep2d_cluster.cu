@@ -1044,7 +1044,7 @@ int c2_remote(int rpc, int N, int R) {
 // estimate, with the bands' split from c2_band_rank, takes on average 2.8 %
 // longer than the best of the measured ones (at most 26 %).  Costs without the
 // remote rows, and without clusters of 4 rows a march: 6.3 % (93 %; 1500 x 60
-// 5.0 us a step instead of 2.8, 601 x 201 4.7 instead of 3.5).
+// 5.0 us a step instead of 3.0, 601 x 201 4.7 instead of 3.6).
 double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band, int c2s) {
   const int units = (rpc + N - 1) / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
   const double u = units / 32.0, order8 = R == 4;

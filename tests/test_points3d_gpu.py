@@ -56,3 +56,44 @@ def test_against_oracle(cuda_lib, case):
         dobs = oracle_dobs(w)
         gf = host(p.gradient_full(to_dev(w.vel0), to_dev(w.wavelet), to_dev(dobs))[0])
         assert rel_l2(gf, oracle.batch_gradient_full(w, w.vel0, dobs)[0]) <= 1e-4
+
+
+def test_many_points_at_a_node(cuda_lib):
+    """Every surface node of a ragged grid several times and one node 300 times,
+    in mixed order, two shots with different multiplicities: adjoint against the
+    oracle, and a repeated call bit for bit."""
+    w = wl.small_3d(nx=70, ny=19, nz=21, nt=30, order=8, nshots=2)
+    rng = np.random.default_rng(11)
+    surf = np.arange(w.nx * w.ny)
+    rec = np.stack([rng.permutation(np.concatenate([surf, surf, surf, np.full(300, 2 * w.nx * w.ny + 67)])),
+                    rng.permutation(np.concatenate([np.repeat(surf[:400], 10), surf[:290]]))]).astype(np.int64)
+    w = dataclasses.replace(w, rec=rec)
+    s = wl.synthetic_data(2, w.nt, rec.shape[1], seed=9)
+    p = problem(w)
+    q = host(p.adjoint(to_dev(w.vel0), to_dev(s)))
+    for k in range(2):
+        assert rel_l2(q[k], oracle.adjoint(oracle.grid_of(w), w.src[k], w.rec[k], w.vel0, s[k])) <= 1e-5, k
+    assert np.array_equal(q, host(p.adjoint(to_dev(w.vel0), to_dev(s))))
+
+
+def test_time_of_doubled_receivers(cuda_lib):
+    """Two receivers at every surface node take two additions a node, not a scan
+    of all shared entries (250 times the call with one receiver a node)."""
+    import torch
+
+    def ms(times):
+        w = wl.small_3d(nx=64, ny=64, nz=64, nt=40, order=8, nshots=1)
+        w = dataclasses.replace(w, rec=np.tile(np.arange(64 * 64, dtype=np.int64), times)[None])
+        p, v = problem(w), to_dev(w.vel0)
+        s = to_dev(wl.synthetic_data(1, w.nt, w.rec.shape[1], seed=9))
+        best = np.inf
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            p.adjoint(v, s)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    assert ms(2) <= 4 * ms(1)
