@@ -308,13 +308,15 @@ tp_status tp_workspace_status(void* ws, size_t ws_bytes, void* stream);
 
 /* Sets the spin limit, in SM clock cycles, of the bounded device-side waits
  * between the roles of the pipelined kernels (the 3-D sweep's copy producer
- * and its consumers) for every launch that follows, process-wide; 0 restores
+ * and its consumers) and between the bands of the 2-D stepping (a CTA waits for
+ * its neighbours' edge rows) for every launch that follows, process-wide; 0 restores
  * the default (2e9 cycles, about one second).  Waits by which a kernel that
  * gives up first lets its own copies land keep the default, so a kernel always
  * exits with nothing in flight.  A limit shorter than a copy's latency makes
  * the waits give up: the calls launched with it set the flag that
  * tp_workspace_status reports as TP_ERR_TIMEOUT, their misfit and gradient
- * norm read NaN, and their other results are invalid.  The paper has no
+ * norm read NaN, and their other results are invalid (2-D: the samples of the
+ * last level that such a launch formed are NaN).  The paper has no
  * counterpart: this exists to exercise the timeout path.  Errors: TP_ERR_ARG
  * (cycles < 0). */
 tp_status tp_set_wait_limit(int64_t cycles);

@@ -35,8 +35,8 @@
 //     carry the step's tag: no fence and no flag (1640-2480 cycles from the store
 //     to the reader; 3100 for a flag behind a fence), and most of that passes
 //     while the rest of the band is marched.  The wait is bounded: on a timeout
-//     the CTA sets bit 0 of *err and steps on without waiting (its results are
-//     then invalid).
+//     the CTA sets bit 0 of *err and steps on without waiting; the launch then
+//     ends with NaN in its last level and samples.
 // Why both: clusters of this size leave SMs idle (8 shots of 12 CTAs: 96 of
 // 152 SMs; 7 clusters of 16 at once), bands use all of them, but an exchange
 // through L2 costs more than a cluster barrier, which decides on small grids;
@@ -985,6 +985,17 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
         *reinterpret_cast<uint2*>(eb + (long long)((lfin - a.dir) & 1) * a.L.field + go) =
             *reinterpret_cast<const uint2*>((a.nsteps & 1 ? E0 : E1) + so);
       }
+    // after a wait that gave up (here or in a neighbour, before its rows came
+    // here): the last level's samples and a node of it are NaN, so that no result
+    // formed from invalid rows passes for a valid one
+    if (BAND && (*aborted || (*static_cast<volatile int*>(a.err) & 1))) {
+      const float nan = __int_as_float(0x7fffffff);
+      if (ns > 0 && a.samp_out && lfin + a.samp_shift >= 0) {
+        float* out = a.samp_out + (long long)shot * a.samp_out_ss + (long long)(lfin + a.samp_shift) * a.nsamp;
+        for (int i = tid; i < ns; i += C2_THREADS) out[sl[i] & 0xffffu] = nan;
+      }
+      if (tid == 0) ring[slot(lfin) + (long long)(z0 + H) * px + HX] = nan;
+    }
     if (!BAND) cluster_wait();  // no CTA leaves (or starts the next shot) while a neighbour reads its band
     __syncthreads();            // this shot's lists and levels are no longer read
   }

@@ -211,8 +211,8 @@ def tp_sweep2d_plan(grid, geom, adjoint: bool = False) -> tuple:
 
 
 def tp_set_wait_limit(cycles: int):
-    """Spin limit (SM cycles) of the pipelined kernels' role waits for the
-    launches that follow; 0 restores the default (about one second)."""
+    """Spin limit (SM cycles) of the pipelined kernels' role waits and of the 2-D bands' waits for
+    their neighbours, for the launches that follow; 0 restores the default (about one second)."""
     _check(lib().tp_set_wait_limit(int(cycles)))
 
 
