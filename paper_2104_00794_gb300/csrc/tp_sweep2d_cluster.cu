@@ -65,6 +65,7 @@
 #include <vector>
 
 #include "tp_internal.h"
+#include "tp_quotient.h"
 
 namespace tp {
 
@@ -178,28 +179,6 @@ __device__ __forceinline__ void st_words(unsigned char* p, uint32_t v0, uint32_t
 
 __device__ __forceinline__ float comp4(const float4& v, int p) {
   return p == 0 ? v.x : (p == 1 ? v.y : (p == 2 ? v.z : v.w));
-}
-
-// n / b, b = 1 + a of the absorbing layer, with inv = 1 / b correctly rounded:
-// two residual corrections give the correctly rounded quotient (Markstein 1990)
-// while the residual does not underflow.  The values ahead of a wave are tiny
-// over most of a layer; they are divided scaled by 2^96, and a subnormal result,
-// then rounded a second time, moves to its other neighbour where the first
-// rounding had made a tie.  (A plain division, with its slow branch for zeros and
-// tiny values, took 13 us of a 17 us step: 601 x 201, 16 shots.)
-__device__ __forceinline__ float quotient(float n, float b, float inv) {
-  const bool tiny = fabsf(n) < 0x1p-60f;
-  if (tiny) n *= 0x1p96f;
-  float q = n * inv;
-  q = fmaf(fmaf(-q, b, n), inv, q);
-  const float r = fmaf(-q, b, n);
-  q = fmaf(r, inv, q);
-  if (tiny) {
-    const float s = q, d = s * 0x1p-96f, diff = fmaf(d, -0x1p96f, s);
-    q = d;
-    if (fabsf(diff) == 0x1p-54f && fmaf(-s, b, n) * diff > 0.f) q += copysignf(0x1p-149f, diff);
-  }
-  return fabsf(n) <= 3.402823466e38f ? q : n;  // infinities and NaN: no residual
 }
 
 // The operators of one row, 4 points: u[i] the rows i - R of the column (u[R]
