@@ -50,7 +50,8 @@
 // neighbours, c2, the previous and the new level, the ring) and by issue.
 //
 // Levels form: the arithmetic of the per-step 2-D sweep, operation for
-// operation (bit-identical results), with or without the absorbing layer.
+// operation (bit-identical results, but for entries that share a node, whose
+// products the per-step path adds unrounded), with or without the absorbing layer.
 // Compensated form (forward only): the wavefield is a double-float u + e (e
 // stored as bf16) stepped with an error-free transformation, so that the
 // rounding of the stored levels, which the Laplacian of the probed field
@@ -1125,7 +1126,7 @@ C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, 
 }
 
 // clusters of C CTAs with `smem` bytes each that fit on the current device at
-// once (cached); without a device, a guess for planning
+// once (cached); without a device, what a GB300 reports
 template <int R, int MODE, int N, bool C2S>
 int c2_max_clusters(int C, size_t smem) {
   static std::mutex m;
@@ -1133,7 +1134,8 @@ int c2_max_clusters(int C, size_t smem) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
-    return std::max(1, C2_MAXBANDS / 2 / C);
+    static const int gb300[C2_MAXC] = {152, 76, 46, 36, 28, 23, 15, 15, 15, 13, 8, 8, 7, 7, 7, 7};
+    return gb300[C - 1];
   }
   const long long key = ((long long)dev << 40) | ((long long)C << 32) | (long long)smem;
   {
