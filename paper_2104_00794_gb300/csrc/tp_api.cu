@@ -265,7 +265,7 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
   if (P->comp && !P->c2d)
     return fail(TP_ERR_ARG, "the compensated form needs a 2-D grid without an absorbing layer whose shot fits one "
                             "thread-block cluster, with at most 1024 sources and receivers per shot");
-  if (P->c2d) P->o_edge = take(cur, edge2d_bytes(P->L, P->W));
+  if (P->c2d) P->o_edge = take(cur, edge2d_bytes(P->L, P->W, P->nshots, P->comp));
   if (P->comp) P->o_e = take(cur, (size_t)2 * ns * P->L.field * 2);  // bf16 low parts, two levels per shot
   if (P->form == TP_FORM_INCREMENT) P->o_w = take(cur, (size_t)ns * fb);  // the increment field of each shot
   switch (op) {
@@ -383,7 +383,7 @@ tp_status setup(const Ctx& c, const tp_grid* g, const tp_geom* geo, const float*
   if (!vel) return fail(TP_ERR_ARG, "vel is NULL");
   TRY(cudaMemsetAsync(c.scal(), 0, SCAL_BYTES, c.st));
   TRY(cudaMemsetAsync(c.at<float>(P.o_c2), 0, P.c2_bytes, c.st));
-  if (P.c2d) TRY(cudaMemsetAsync(c.at<char>(P.o_edge), 0, edge2d_bytes(P.L, P.W), c.st));
+  if (P.c2d) TRY(cudaMemsetAsync(c.at<char>(P.o_edge), 0, edge2d_bytes(P.L, P.W, P.nshots, P.comp), c.st));
   const double dt2 = (double)g->dt * (double)g->dt;
   TRY(launch_prep_c2(P.L, vel, dt2 / ((double)g->h * (double)g->h), c.at<float>(P.o_c2), c.st));
   TRY(launch_prep_points(P.L, P.W, geo->src, (long long)P.nshots * P.nsrc, vel, dt2, c.at<long long>(P.o_soff),

@@ -202,7 +202,7 @@ bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int
 // whether the levels form (with or without an absorbing layer) can run on
 // bands of the whole GPU
 bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec);
-size_t edge2d_bytes(const Layout& L, const Weights& W);
+size_t edge2d_bytes(const Layout& L, const Weights& W, int nshots, bool comp);  // of any plan
 // the split that launch_cluster2d takes on the current device (tp_sweep2d_plan)
 void plan2d(const Layout& L, const Weights& W, bool comp, int nshots, int ninj, int nsamp, int plan[6]);
 

@@ -1264,8 +1264,9 @@ void plan2d(const Layout& L, const Weights& W, bool comp, int nshots, int ninj, 
   std::copy(v, v + 6, plan);
 }
 
-size_t edge2d_bytes(const Layout& L, const Weights& W) {
-  return (size_t)C2_MAXBANDS * 4 * W.R * ((L.nx + 3) / 4) * 16 * 3;
+size_t edge2d_bytes(const Layout& L, const Weights& W, int nshots, bool comp) {
+  const long long ctas = std::min<long long>(C2_MAXBANDS, (long long)nshots * ((L.nz + 7) / 8));  // bands have 8 rows at least
+  return (size_t)ctas * 4 * W.R * ((L.nx + 3) / 4) * 16 * (comp ? 3 : 2);
 }
 
 cudaError_t launch_cluster2d(const Cluster2dArgs& c, cudaStream_t s) {
