@@ -260,7 +260,7 @@ tp_status make_plan(int op, const tp_grid* g, const tp_geom* geo, const tp_probe
   P->o_c2 = take(cur, P->c2_bytes);
   P->form = g->form;
   P->comp = g->form == TP_FORM_COMPENSATED;
-  P->c2d = P->comp ? cluster2d_fits(P->L, P->W, P->nshots, P->nsrc, P->nrec, true)
+  P->c2d = P->comp ? compensated2d_fits(P->L, P->W, P->nsrc, P->nrec)
                    : g->form == TP_FORM_LEVELS && persist2d_fits(P->L, P->W, P->nshots, P->nsrc, P->nrec);
   if (P->comp && !P->c2d)
     return fail(TP_ERR_ARG, "the compensated form needs a 2-D grid without an absorbing layer whose shot fits one "
@@ -630,7 +630,7 @@ tp_status tp_form_supported(const tp_grid* grid, const tp_geom* geom) {
     const Layout L = make_layout(grid->ndim, grid->nx, grid->ny, grid->nz);
     Weights W = stencil_weights(grid->order);
     W.sw = grid->sponge_eta > 0.f ? grid->sponge : 0;
-    if (!cluster2d_fits(L, W, geom->nshots, geom->nsrc, geom->nrec, true))
+    if (!compensated2d_fits(L, W, geom->nsrc, geom->nrec))
       return fail(TP_ERR_ARG, "the compensated form needs a 2-D grid without an absorbing layer whose shot fits one "
                               "thread-block cluster, with at most 1024 sources and receivers per shot");
   }

@@ -198,7 +198,7 @@ struct Cluster2dArgs {
 cudaError_t launch_cluster2d(const Cluster2dArgs& a, cudaStream_t s);
 // whether a shot of this grid fits one thread-block cluster (2-D, no absorbing
 // layer, at most 1024 sources and receivers): the compensated form's condition
-bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec, bool comp);
+bool compensated2d_fits(const Layout& L, const Weights& W, int nsrc, int nrec);
 // whether the levels form (with or without an absorbing layer) can run on
 // bands of the whole GPU
 bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec);

@@ -1002,11 +1002,11 @@ size_t c2_bytes(int rpc, int N, int sx, int nx4, int R, int mode, bool band, boo
 // of the compensated form: an upper bound of what a lean cluster of these CTAs
 // needs (c2_bytes without c2: at least 32 rpc + 32 R + 2 cap - 40 bytes less), so
 // that every grid accepted has a plan.
-bool c2_accepts(const Layout& L, int R, int C, bool comp, int cap) {
+bool c2_accepts(const Layout& L, int R, int C, int cap) {
   const int nx4 = (L.nx + 3) / 4, sx = 4 * nx4 + 8;
   const int rpc = (L.nz + C - 1) / C;
   if (nx4 > C2_MAXCOL) return false;
-  size_t b = (size_t)(2 * rpc + 1) * sx * 4 + (comp ? (size_t)2 * rpc * sx * 2 : 0);
+  size_t b = (size_t)(2 * rpc + 1) * sx * 4 + (size_t)2 * rpc * sx * 2;
   b += (size_t)2 * 2 * (rpc + 2 * R) * sizeof(void*) + (size_t)cap * 20 + (size_t)(4 + C2_THREADS / 32) * 4;
   return (b + 15) / 16 * 16 <= C2_SMEM;
 }
@@ -1241,14 +1241,13 @@ cudaError_t c2_launch(const C2Args& a0, cudaStream_t s) {
 
 }  // namespace
 
-bool cluster2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec, bool comp) {
-  (void)nshots;
+bool compensated2d_fits(const Layout& L, const Weights& W, int nsrc, int nrec) {
   if (L.ndim != 2 || W.sw > 0) return false;
   if (nsrc > C2_MAXLIST || nrec > C2_MAXLIST) return false;
   // the larger of the two sets in both lists covers the forward and the adjoint launches
   const int cap = c2_cap(std::max(nsrc, nrec));
   for (int C = 1; C <= C2_MAXC; ++C)
-    if (c2_accepts(L, W.R, C, comp, cap)) return true;
+    if (c2_accepts(L, W.R, C, cap)) return true;
   return false;
 }
 

@@ -372,7 +372,6 @@ sweep3d_tma(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUte
   const int tx = tid % (BX / 4), ty = tid / (BX / 4), lane = tid & 31;
   constexpr int RW = C::UW / 4;  // float4 per staged row
   constexpr bool POINTS = MODE != MODE_IMAGE;
-  constexpr int UNROLL = (MODE != MODE_INC && !DAMP) ? 2 * R + 1 : 1;
   const float4* U4 = reinterpret_cast<const float4*>(sU);
   const float4* I4 = reinterpret_cast<const float4*>(sI);
   uint32_t ku = 0, kp = 0;
