@@ -39,13 +39,15 @@
 //     ends with NaN in its last level and samples.
 // Why both: clusters of this size leave SMs idle (8 shots of 12 CTAs: 96 of
 // 152 SMs; 7 clusters of 16 at once), bands use all of them, but an exchange
-// through L2 costs more than a cluster barrier, which decides on small grids;
-// c2_step_cost has the measurements.
-// Measured per step on GB300, before (clusters only, one CTA of 16 warps with
-// guarded rows) and now: 601 x 201, 16 shots, order 8: levels 6.8 -> 3.9 us,
-// compensated 12.6 -> 8.1 us; 801 x 301, 8 shots: 7.1 -> 3.9, 18.6 -> 8.0 us; 101
-// x 101, one shot, order 4: 2.0 -> 1.5 us; an absorbing layer (601 x 201, 4
-// shots, then two launches per step) 29 -> 4.6 us.  Bound by the shared memory
+// through L2 costs more than a cluster barrier, which decides on small grids and
+// on wide, shallow ones (clusters of four rows a march); c2_step_cost has the
+// measurements.
+// Measured per step on GB300 (forward calls of 1500 and 300 levels, their
+// difference), before (clusters only, one CTA of 16 warps with guarded rows) and
+// now: 601 x 201, 16 shots, order 8: levels 6.1 -> 3.6 us, compensated 13.2 ->
+// 7.8 us; 801 x 301, 8 shots: 6.4 -> 3.6, 19.7 -> 8.2 us; 101 x 101, one shot,
+// order 4: 1.7 -> 1.25 us; an absorbing layer (601 x 201, 4 shots, then two
+// launches per step) 31 -> 4.2 us.  Bound by the shared memory
 // pipe (32 wavefronts per 128 points of the levels form: the row and its
 // neighbours, c2, the previous and the new level, the ring) and by issue.
 //
@@ -311,8 +313,8 @@ __device__ __forceinline__ void row4(const Weights& W, const float4* u, Low low,
 // LEAN (clusters without c2 in shared memory, for wide grids): the levels alone
 // fill the shared memory.  c2 comes from global memory, nothing is kept per
 // unit, all entries are added after the march, and the last chunk of a band
-// has as many rows as are left.  Compensated step, order 8: 1800 x 100 9.3 us,
-// 2001 x 101 x 8 shots 11.5 us (8.9 and 17.7 us when a cluster kept c2 in global
+// has as many rows as are left.  Compensated step, order 8: 1800 x 100 8.6 us,
+// 2001 x 101 x 8 shots 10.9 us (8.3 and 17.1 us when a cluster kept c2 in global
 // memory and guarded every row).
 template <int R, int MODE, bool BAND, int N, bool C2S>
 __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
@@ -353,9 +355,9 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   // points; else (a chain) entries by node: those in edge rows are walked along
   // nxt when the unit is marched, the others are added after the march, where
   // an entry with LEAD stands for the nxt entries of its node from it on.  Step
-  // at 401 x 401 with 1024 receivers at a node 10.7 us, in a patch of 32 x 32
-  // 5.8 us, in a row 4.0 us (14 ms, 43 us, 4.0 us when the unit's thread walked
-  // the chain once for every entry).
+  // at 401 x 401 with 1024 receivers at a node 9.8 us, in a patch of 32 x 32
+  // 5.7 us, along a borehole 4.4 us, in a row 3.5 us (14 ms, 43, 7.5 and 4.0 us
+  // when the unit's thread walked the chain once for every entry).
   // Per unit, read where it is used (kept in registers, it spilled):
   //   ua[u]: byte offset of its first row in a level buffer, offset in a field,
   //          byte offset in c2, flags | its first row << 8
@@ -1032,10 +1034,10 @@ int c2_remote(int rpc, int N, int R) {
 // memory.  The coefficients are a least-squares fit (relative, non-negative) to
 // 9686 measured splits of 260 random grids (8 to 2048 x 16 to 420, 1 to 40 shots,
 // both orders, all modes); mean error 3 to 8 %.  The split with the least
-// estimate, with the bands' split from c2_band_rank, takes on average 2.8 %
+// estimate, with the bands' split from c2_band_rank, takes on average 2.4 %
 // longer than the best of the measured ones (at most 26 %).  Costs without the
 // remote rows, and without clusters of 4 rows a march: 6.3 % (93 %; 1500 x 60
-// 5.0 us a step instead of 3.0, 601 x 201 4.7 instead of 3.6).
+// 5.0 us a step instead of 2.7, 601 x 201 4.3 instead of 3.2).
 double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band, int c2s) {
   const int units = (rpc + N - 1) / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
   const double u = units / 32.0, order8 = R == 4;
