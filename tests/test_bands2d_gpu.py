@@ -187,3 +187,45 @@ def test_launch_per_step_against_oracle(sponge):
     spec = api.ProbeSpec(kind="rademacher", r=4, T=32, seed=w.seed)
     ref, _ = oracle.batch_gradient_probed(w, w.vel0, dobs, kind="rademacher", r=4, seed=w.seed)
     assert rel_l2(host(p.gradient_probed(*args, spec)[0]), ref) <= 1e-4
+
+
+KINDS = [  # nx, nz, shots, order, sponge, form -> bands (1) or clusters (2), rows per march, c2 in shared memory
+    (1001, 17, 1, 4, 0, "compensated", 2, 2, 1), (1300, 41, 1, 4, 0, "compensated", 2, 4, 0),
+    (1300, 100, 1, 4, 0, "compensated", 2, 4, 1), (401, 17, 1, 8, 0, "compensated", 2, 2, 1),
+    (1500, 41, 1, 8, 0, "compensated", 2, 4, 0), (1001, 41, 1, 8, 0, "compensated", 2, 4, 1),
+    (1500, 150, 1, 8, 0, "compensated", 1, 4, 0), (1500, 150, 1, 4, 0, "compensated", 1, 4, 0),
+    (1001, 17, 1, 4, 0, "levels", 2, 2, 1), (1800, 41, 2, 4, 0, "levels", 2, 4, 0), (1300, 41, 3, 4, 0, "levels", 2, 4, 1),
+    (401, 17, 9, 8, 0, "levels", 2, 2, 1), (1300, 41, 1, 8, 0, "levels", 2, 4, 0), (1001, 41, 1, 8, 0, "levels", 2, 4, 1),
+    (2045, 150, 1, 8, 0, "levels", 1, 4, 0), (2045, 150, 1, 4, 0, "levels", 1, 4, 0), (2045, 100, 1, 8, 10, "levels", 1, 4, 0),
+    (2045, 100, 1, 4, 10, "levels", 1, 4, 0), (1300, 17, 1, 8, 10, "levels", 2, 2, 1), (1500, 41, 1, 8, 10, "levels", 2, 4, 1),
+    (1300, 17, 1, 4, 10, "levels", 2, 2, 1),
+]
+
+
+@pytest.mark.parametrize("kind", KINDS, ids=lambda c: "x".join(map(str, c)))
+def test_every_kind_of_split_against_oracle(kind):
+    """Wide grids, where the planner takes the marches and the places of c2 that the
+    other tests do not: clusters of two and four rows a march, lean ones, bands
+    with c2 in global memory; points beside the CTAs' edges, in a patch, in a row."""
+    nx, nz, shots, order, sponge, form, *want = kind
+    w = wl.small_2d(nx=nx, nz=nz, nt=41, order=order, nshots=shots)
+    if sponge:
+        w = wl.with_sponge(w, sponge)
+    w = at_band_edges(w, 4)
+    pl = plan(w, form)
+    assert [pl[0], pl[3], pl[5]] == want, pl
+    patch = ((np.arange(5, 13)[:, None] % nz) * nx + nx // 2 + np.arange(9)).ravel()
+    row = 3 * nx + np.arange(nx // 2 - 40, nx // 2 + 40)
+    w = dataclasses.replace(w, rec=np.concatenate([w.rec, np.tile(np.concatenate([patch, row]), (shots, 1))], axis=1))
+    p = problem(w, form=form)
+    d = host(p.forward(to_dev(w.vel_true), to_dev(w.wavelet)))
+    assert rel_l2(d, oracle.batch_forward(w, w.vel_true)) <= 1e-5
+    s = wl.synthetic_data(shots, w.nt, w.rec.shape[1], seed=9)
+    q = host(p.adjoint(to_dev(w.vel0), to_dev(s)))
+    for k in range(shots):
+        assert rel_l2(q[k], oracle.adjoint(oracle.grid_of(w), w.src[k], w.rec[k], w.vel0, s[k])) <= 1e-5, k
+    back = dataclasses.replace(w, src=w.rec, rec=w.src,
+                               wavelet=np.ascontiguousarray(np.repeat(w.wavelet[:, :, :1], w.rec.shape[1], axis=2)))
+    if form == "compensated":  # the points inject in the compensated form too
+        d = host(problem(back, form=form).forward(to_dev(w.vel_true), to_dev(back.wavelet)))
+        assert rel_l2(d, oracle.batch_forward(back, w.vel_true)) <= 1e-5
