@@ -1017,7 +1017,7 @@ struct C2Plan {
   int C = 0, rpc = 0, N = 0, groups = 0, c2s = 0;  // CTAs per shot, rows per CTA and unit, shots at once
   bool band = false;
   size_t smem = 0;
-  double est = 0;
+  double est = 0, rank = 0;  // c2_step_cost and c2_rank, all rounds
 };
 
 // rows that the marches of a column read from neighbouring CTAs
@@ -1029,54 +1029,53 @@ int c2_remote(int rpc, int N, int R) {
 
 // Estimated us of a step in which every CTA has rpc rows, marched N at a time
 // (rows of nx4 columns, units of 32 per warp): a sum of the rows marched, the
-// 2R queue rows that every march fills, the passes of the CTA's threads, a
-// march's latency and, in clusters, the rows read from a neighbour's shared
-// memory.  The coefficients are a least-squares fit (relative, non-negative) to
-// 9686 measured splits of 260 random grids (8 to 2048 x 16 to 420, 1 to 40 shots,
-// both orders, all modes); mean error 3 to 8 %.  The split with the least
-// estimate, with the bands' split from c2_band_rank, takes on average 2.4 %
-// longer than the best of the measured ones (at most 26 %).  Costs without the
-// remote rows, and without clusters of 4 rows a march: 6.3 % (93 %; 1500 x 60
-// 5.0 us a step instead of 2.7, 601 x 201 4.3 instead of 3.2).
+// 2R queue rows that every march fills, the passes of the CTA's threads, their
+// latency (by rows of a march) and, in clusters, the rows read from a neighbour's
+// shared memory.  The coefficients are a least-squares fit (relative,
+// non-negative) to 19036 measured splits of 480 random grids (8 to 2048 x 16 to
+// 420, 1 to 128 shots, both orders, all modes); mean error 4 to 9 %.
 double c2_step_cost(int rpc, int N, int nx4, int R, int mode, bool band, int c2s) {
   const int units = (rpc + N - 1) / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
   const double u = units / 32.0, order8 = R == 4;
   if (band) {
     // [mode]: constant, order 8, warps, latency by N, columns, passes, rows (N = 8), rows (c2 in global memory), rows (order 8)
-    static const double K[3][9] = {{1.176, 1.122, 0., 0., 0.306, 0.660, 0.0061, 0.0058, 0.0005},
-                                   {0.033, 0.869, 0.0472, 0.170, 0.336, 1.273, 0.0096, 0.0051, 0.0144},
-                                   {0., 0.922, 0.0395, 0.411, 0.108, 1.175, 0.0075, 0.0058, 0.0064}};
+    static const double K[3][9] = {{1.011, 1.058, 0.0056, 0.0115, 0.318, 0.669, 0.0062, 0.0054, 0.0006},
+                                   {0., 0.808, 0.0481, 0.166, 0.264, 1.318, 0.0106, 0.0054, 0.0146},
+                                   {0., 0.833, 0.0454, 0.442, 0.082, 1.023, 0.0064, 0.0069, 0.0070}};
     const double* k = K[mode];
     return k[0] + k[1] * order8 + k[2] * u + k[3] * N + k[4] * nx4 / 100 + k[5] * passes +
            u * N * (k[6] * (N == 8) + k[7] * !c2s + k[8] * order8);
   }
-  if (!c2s) {  // lean: constant, order 8, rows filled, passes, remote rows
-    static const double K[2][5] = {{1.487, 0.139, 0.0053, 0.907, 0.0037}, {1.362, 0.611, 0.0161, 1.330, 0.}};
+  if (!c2s) {  // lean: constant, order 8, rows filled, passes
+    static const double K[2][4] = {{1.392, 0.169, 0.0051, 0.953}, {1.086, 0.662, 0.0142, 1.594}};
     const double* k = K[mode];
-    return k[0] + k[1] * order8 + k[2] * u * 2 * R + k[3] * passes + k[4] * c2_remote(rpc, N, R) * nx4 / 1000;
+    return k[0] + k[1] * order8 + k[2] * u * 2 * R + k[3] * passes;
   }
-  // clusters, [mode]: constant, order 8, rows marched, rows filled, remote rows, latency by N, passes
-  static const double K[3][7] = {{0.964, 0.259, 0.0103, 0.0023, 0.137, 0.133, 0.325},
-                                 {0.899, 0.428, 0.0227, 0.0048, 0.224, 0.241, 0.346},
-                                 {0.912, 0.263, 0.0206, 0.0006, 0.128, 0.348, 0.480}};
+  // clusters, [mode]: constant, order 8, rows marched, rows filled, remote rows, latency by N, passes, latency by N of a pass
+  static const double K[3][8] = {{1.075, 0.229, 0.0053, 0.0030, 0.125, 0., 0.168, 0.155},
+                                 {1.108, 0.374, 0.0155, 0.0057, 0.192, 0., 0.085, 0.267},
+                                 {1.271, 0.149, 0.0108, 0.0021, 0.087, 0.0595, 0.145, 0.322}};
   const double* k = K[mode];
   return k[0] + k[1] * order8 + k[2] * u * N + k[3] * u * 2 * R + k[4] * c2_remote(rpc, N, R) * nx4 / 1000 + k[5] * N +
-         k[6] * passes;
+         passes * (k[6] + k[7] * N);
 }
 
-// Rank of a split into bands among splits into bands: a step's time with the
-// floor that the exchange sets (3.6 us at order 8).  Near the floor the phases of
-// the exchange decide, by up to 25 % and not smoothly; the fit above has no
-// floor and picked shorter marches there (601 x 201 x 16 shots 4.2 us instead of
-// 3.9, 397 x 401 x 4 3.8 instead of 3.1), but it tells the splits at the floor
-// apart (601 x 201: 26 bands of 8 rows 3.5 us, 13 of 16 4.1): a fifth of it counts.
-// (With a layer the marches are longer and the fit alone ranks better.)
-double c2_band_rank(int rpc, int N, int nx4, int R, int mode) {
+// Rank of a split into bands, or into clusters of one or two rows a march: a
+// step's time from measurements of medium grids, with the floor that the
+// exchange of bands sets.  Near the floor the phases of the exchange decide, by
+// up to 25 % and not smoothly, where the fit above is no better (by the fit alone:
+// 601 x 201 x 16 shots 4.2 us instead of 3.9, 397 x 401 x 4 3.8 instead of 3.1); it
+// knows no remote rows (c2_choose).
+double c2_rank(int rpc, int N, int nx4, int R, int mode, bool band) {
   const int units = rpc / N * nx4, passes = (units + C2_THREADS - 1) / C2_THREADS;
   const double w = std::min(16, (units + 31) / 32);
-  const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : 0.0185;
-  const double floor = R == 4 ? 3.6 : (N == 8 ? 1.9 : 1.5) * (mode == C2_COMP ? 1.45 : 1.0);
-  return std::max(floor, (mode == C2_COMP ? 1.9 : 1.6) + passes * N * row * w) + 0.03 * passes * w;
+  if (band) {
+    const double row = mode == C2_COMP ? (N == 8 ? 0.066 : 0.05) : (mode == C2_DAMP ? 0.026 : 0.0185);
+    const double floor = R == 4 ? 3.6 : (N == 8 ? 1.9 : 1.5) * (mode == C2_COMP ? 1.45 : 1.0);
+    return std::max(floor, (mode == C2_COMP ? 1.9 : 1.6) + passes * N * row * w) + 0.03 * passes * w;
+  }
+  const double row = mode == C2_COMP ? 0.05 : (mode == C2_DAMP ? 0.024 : 0.02), fill = mode == C2_COMP ? 0.004 : 0.0025;
+  return (N == 1 ? 1.25 : 1.4) + passes * w * (N * row + 2 * R * fill);
 }
 
 // c2s 0: c2 in global memory (bands; lean clusters)
@@ -1093,7 +1092,9 @@ C2Plan c2_try(const Layout& L, int R, int mode, int sw, int nshots, int C, int N
   const size_t sm = c2_bytes(rpc, N, sx, nx4, R, mode, band, c2s, sw, capi, caps);
   if (sm > C2_SMEM) return p;
   p.C = C; p.rpc = rpc; p.N = N; p.groups = std::min(groups, nshots); p.c2s = c2s; p.band = band; p.smem = sm;
-  p.est = (double)((nshots + p.groups - 1) / p.groups) * c2_step_cost(rpc, N, nx4, R, mode, band, c2s);
+  const double rounds = (nshots + p.groups - 1) / p.groups;
+  p.est = rounds * c2_step_cost(rpc, N, nx4, R, mode, band, c2s);
+  p.rank = rounds * c2_rank(rpc, N, nx4, R, mode, band);
   return p;
 }
 
@@ -1107,23 +1108,24 @@ int c2_sms() {
   return std::min(sms, C2_MAXBANDS);
 }
 
-// The best split into bands of one cooperative grid (C = 0: none fits)
-C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, int caps) {
-  C2Plan best;
-  double least = 0;
-  const int sms = c2_sms();
-  for (int C = 1; C <= sms; ++C)
+// The best split into bands of one cooperative grid (C = 0: none fits), by rank;
+// fit (may be null): with a fifth of the estimate, which tells the splits at the
+// floor apart (601 x 201: 26 bands of 8 rows 3.2 us, 13 of 16 4.1).  With a layer,
+// whose marches are longer, both by the estimate (order 4, 601 x 201 x 16: 5.3 us,
+// by rank 5.9).
+C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, int caps, C2Plan* fit) {
+  C2Plan best, other;
+  auto rank = [&](const C2Plan& p) { return mode == C2_DAMP ? p.est : p.rank; };
+  const int sms = c2_sms(), most = std::min(sms, (L.nz + 7) / 8);  // (bands have 8 rows at least)
+  for (int C = 1; C <= most; ++C)
     for (int N : {8, 4}) {
       C2Plan p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 1, capi, caps);
       if (!p.C) p = c2_try(L, R, mode, sw, nshots, C, N, sms / C, true, 0, capi, caps);
       if (!p.C) continue;
-      const double rounds = (nshots + p.groups - 1) / p.groups;
-      const double rank =
-          mode == C2_DAMP ? p.est : rounds * c2_band_rank(p.rpc, N, (L.nx + 3) / 4, R, mode) + 0.2 * p.est;
-      if (best.C && rank >= least) continue;
-      best = p;
-      least = rank;
+      if (!best.C || rank(p) < rank(best)) best = p;
+      if (!other.C || rank(p) + 0.2 * p.est < rank(other) + 0.2 * other.est) other = p;
     }
+  if (fit) *fit = other;
   return best;
 }
 
@@ -1167,14 +1169,22 @@ int c2_max_clusters(int C, size_t smem) {
   return n;
 }
 
+// The split of the least rank among bands and clusters of one and two rows a
+// march; another one (clusters of four rows and lean ones included) where the
+// fitted estimate gives it 10 % less.  Over the 480 grids no split chosen so is
+// more than 3 % slower than the one by rank alone and 52 are faster by more (1500 x
+// 60 2.7 us a step instead of 5.0, 601 x 201 3.2 instead of 4.3, 2000 x 64 x 2 3.3
+// instead of 4.4); by the estimate alone 13 and 104.  The chosen split takes on
+// average 3.0 % longer than the best measured one (by rank 5.0 %).
 template <int R, int MODE>
 C2Plan c2_choose(const Layout& L, int sw, int nshots, int capi, int caps) {
-  C2Plan best = c2_bands(L, R, MODE, sw, nshots, capi, caps);
+  C2Plan best, base = c2_bands(L, R, MODE, sw, nshots, capi, caps, &best);
   auto cluster = [&](int C, int N, int c2s, auto at_once) {
     C2Plan p = c2_try(L, R, MODE, sw, nshots, C, N, nshots, false, c2s, capi, caps);
     if (!p.C) return;
     p = c2_try(L, R, MODE, sw, nshots, C, N, at_once(C, p.smem), false, c2s, capi, caps);
     if (p.C && (!best.C || p.est < best.est)) best = p;
+    if (p.C && N <= 2 && (!base.C || p.rank < base.rank)) base = p;
   };
   for (int C = 1; C <= C2_MAXC; ++C) {
     cluster(C, 4, 1, c2_max_clusters<R, MODE, 4, true>);
@@ -1182,7 +1192,7 @@ C2Plan c2_choose(const Layout& L, int sw, int nshots, int capi, int caps) {
     cluster(C, 1, 1, c2_max_clusters<R, MODE, 1, true>);
     if constexpr (MODE != C2_DAMP) cluster(C, 4, 0, c2_max_clusters<R, MODE, 4, false>);
   }
-  return best;
+  return !base.C || best.est < 0.9 * base.est ? best : base;
 }
 
 template <int R, int MODE, bool BAND, int N, bool C2S>
@@ -1256,7 +1266,7 @@ bool compensated2d_fits(const Layout& L, const Weights& W, int nsrc, int nrec) {
 bool persist2d_fits(const Layout& L, const Weights& W, int nshots, int nsrc, int nrec) {
   if (L.ndim != 2 || nsrc > C2_MAXLIST || nrec > C2_MAXLIST) return false;
   const int cap = c2_cap(std::max(nsrc, nrec));
-  return c2_bands(L, W.R, W.sw > 0 ? C2_DAMP : C2_LEVELS, W.sw, nshots, cap, cap).C > 0;
+  return c2_bands(L, W.R, W.sw > 0 ? C2_DAMP : C2_LEVELS, W.sw, nshots, cap, cap, nullptr).C > 0;
 }
 
 void plan2d(const Layout& L, const Weights& W, bool comp, int nshots, int ninj, int nsamp, int plan[6]) {

@@ -190,15 +190,14 @@ def test_launch_per_step_against_oracle(sponge):
 
 
 KINDS = [  # nx, nz, shots, order, sponge, form -> bands (1) or clusters (2), rows per march, c2 in shared memory
-    (1001, 17, 1, 4, 0, "compensated", 2, 2, 1), (1300, 41, 1, 4, 0, "compensated", 2, 4, 0),
-    (1300, 100, 1, 4, 0, "compensated", 2, 4, 1), (401, 17, 1, 8, 0, "compensated", 2, 2, 1),
-    (1500, 41, 1, 8, 0, "compensated", 2, 4, 0), (1001, 41, 1, 8, 0, "compensated", 2, 4, 1),
-    (1500, 150, 1, 8, 0, "compensated", 1, 4, 0), (1500, 150, 1, 4, 0, "compensated", 1, 4, 0),
-    (1001, 17, 1, 4, 0, "levels", 2, 2, 1), (1800, 41, 2, 4, 0, "levels", 2, 4, 0), (1300, 41, 3, 4, 0, "levels", 2, 4, 1),
-    (401, 17, 9, 8, 0, "levels", 2, 2, 1), (1300, 41, 1, 8, 0, "levels", 2, 4, 0), (1001, 41, 1, 8, 0, "levels", 2, 4, 1),
-    (2045, 150, 1, 8, 0, "levels", 1, 4, 0), (2045, 150, 1, 4, 0, "levels", 1, 4, 0), (2045, 100, 1, 8, 10, "levels", 1, 4, 0),
-    (2045, 100, 1, 4, 10, "levels", 1, 4, 0), (1300, 17, 1, 8, 10, "levels", 2, 2, 1), (1500, 41, 1, 8, 10, "levels", 2, 4, 1),
-    (1300, 17, 1, 4, 10, "levels", 2, 2, 1),
+    (1300, 17, 1, 4, 0, "compensated", 2, 2, 1), (1500, 41, 1, 4, 0, "compensated", 2, 4, 0),
+    (1500, 100, 1, 4, 0, "compensated", 1, 4, 0), (601, 17, 1, 8, 0, "compensated", 2, 2, 1),
+    (1800, 77, 1, 8, 0, "compensated", 2, 4, 0), (1300, 41, 1, 8, 0, "compensated", 2, 4, 1),
+    (1500, 150, 1, 8, 0, "compensated", 1, 4, 0), (1300, 17, 1, 4, 0, "levels", 2, 2, 1),
+    (2045, 100, 1, 4, 0, "levels", 2, 4, 0), (1500, 41, 3, 4, 0, "levels", 2, 4, 1), (2045, 150, 1, 4, 0, "levels", 1, 4, 0),
+    (1001, 17, 9, 8, 0, "levels", 2, 2, 1), (1500, 41, 1, 8, 0, "levels", 2, 4, 0), (1300, 41, 1, 8, 0, "levels", 2, 4, 1),
+    (2045, 150, 1, 8, 0, "levels", 1, 4, 0), (2045, 100, 1, 8, 10, "levels", 1, 4, 0), (2045, 100, 1, 4, 10, "levels", 1, 4, 0),
+    (1001, 17, 1, 8, 10, "levels", 2, 2, 1), (601, 100, 1, 8, 10, "levels", 2, 4, 1), (1300, 17, 1, 4, 10, "levels", 2, 2, 1),
 ]
 
 
