@@ -18,9 +18,9 @@
 //     the rows that a neighbour needs are formed first;
 //   * entries that inject are added in index order at every node
 //     (deterministic): a unit whose entries are one row with one entry per point
-//     at most (a source, surface receivers) and those of the rows next to a
-//     neighbour by the thread that marches the unit, all others after the march,
-//     a thread per node;
+//     at most (a source, surface receivers), those of the rows next to a
+//     neighbour and all of a cluster's by the thread that marches the unit, the
+//     others after the march, a thread per node;
 //   * the levels that the caller needs go to their ring slots in global memory
 //     (the window GEMM reads them, the next launch starts from them).
 // Two exchanges of the band edges (the R rows next to a neighbour):
@@ -64,7 +64,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 #include <vector>
 
 #include "tp_internal.h"
@@ -346,18 +345,19 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   if (COMP) pf = reinterpret_cast<float*>(E1 + (size_t)(rpc + er) * sx);
   float* const c2b = pf;
   if (C2S) pf += (size_t)rpc * 4 * nx4;
-  uint32_t* const il = reinterpret_cast<uint32_t*>(pf);  // injection, by node: node (band index) << 16 | LEAD | k
+  uint32_t* const il = reinterpret_cast<uint32_t*>(pf);  // injection, by node: node (band index) << 16 | LEAD | MANY | k
   uint32_t* const sl = il + a.capi;                      // sampling: the same
   const int vstep = a.capi + 4;                               // floats from one step's values to the next step's
   float* const ival = reinterpret_cast<float*>(sl + a.caps);  // [2][vstep]: values of this step and the next, [capi]: 0
   // entries by unit: in the common case (one row of the unit, one entry per
   // point at most) the row's place in the march and the entry of each of its 4
-  // points; else (a chain) entries by node: those in edge rows are walked along
-  // nxt when the unit is marched, the others are added after the march, where
-  // an entry with LEAD stands for the nxt entries of its node from it on.  Step
-  // at 401 x 401 with 1024 receivers at a node 9.8 us, in a patch of 32 x 32
-  // 5.7 us, along a borehole 4.4 us, in a row 3.5 us (14 ms, 43, 7.5 and 4.0 us
-  // when the unit's thread walked the chain once for every entry).
+  // points; else (a chain) entries by node.  Those in edge rows (WALK: all) are
+  // walked along nxt when the unit is marched; the others are added after the
+  // march, where an entry with LEAD stands for the nxt entries of its node from
+  // it on.  (WALK: so does one with MANY, and the last of them leads on.)  Step at
+  // 401 x 401 with 1024 receivers at a node 9.8 us, in a patch of 32 x 32 5.7 us,
+  // along a borehole 4.4 us, in a row 3.5 us (14 ms, 43, 7.5 and 4.0 us when the
+  // unit's thread walked the chain once for every entry).
   // Per unit, read where it is used (kept in registers, it spilled):
   //   ua[u]: byte offset of its first row in a level buffer, offset in a field,
   //          byte offset in c2, flags | its first row << 8
@@ -368,14 +368,16 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   int4* const ub_ = ua_ + ntab;
   ushort4* const uline = reinterpret_cast<ushort4*>(ub_ + ntab);
   uint16_t* const tl = reinterpret_cast<uint16_t*>(uline + ntab);  // last entry of a unit (set-up)
-  uint16_t* const nxt = tl + (ntab + 1) / 2 * 2;                // next entry of the same unit; LEAD: entries of its node
+  uint16_t* const nxt = tl + (ntab + 1) / 2 * 2;                // next entry of the same unit; LEAD, MANY: entries of its node
   int* const cnt = reinterpret_cast<int*>(nxt + (ntab + 1) / 2 % 2 * 2 + a.capi);  // [0] injection, [1] sampling entries, [3] LEAD used, [4 ..] per-warp counts
   volatile int* const aborted = cnt + 2;
   uint32_t* const tab = reinterpret_cast<uint32_t*>(cnt + 4 + C2_THREADS / 32);  // clusters: edge rows of the levels, low parts
   float2* const dmp = reinterpret_cast<float2*>(tab + (BAND ? 0 : 8 * R));
-  // all chains walked: beside these two marches the code after the march cost a step 6 to 11 %
-  constexpr bool WALK = BAND && (DAMP || !C2S);
-  constexpr uint32_t NONE = 0xffff, LEAD = 0x8000, KMASK = 0x7fff;
+  // all chains walked: beside the marches of clusters, of the layer and of c2 in
+  // global memory the code after the march cost a step 3 to 11 %
+  constexpr bool WALK = !LEAN && (!BAND || DAMP || !C2S);
+  constexpr uint32_t NONE = 0xffff, LEAD = 0x8000, MANY = 0x4000, KMASK = 0x3fff;
+  static_assert(C2_MAXLIST <= (int)KMASK, "an entry's index and two flags in 16 bits");
   constexpr int F_ON = 1, F_UP = 2, F_FULL = 4, F_NB = 8, F_OUT = 16, F_PUB = 32, F_LATE = 64;  // flags of a unit
 
   if (!BAND) {
@@ -560,6 +562,10 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
           if (WALK || (edge && ((int)(l / (uint32_t)sx) - start) * d < R)) {
             if (head == NONE) head = lead;
             last = tail;
+            if (WALK && n > 1) {
+              il[lead] |= MANY;
+              nxt[lead] = (uint16_t)n;
+            }
           } else {
             il[lead] |= LEAD;
             nxt[lead] = (uint16_t)n;
@@ -680,253 +686,220 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
     };
     ask_ahead(tagb);
     const uint32_t sLead = sa(cnt + 3);
-    // The steps.  POINTS: with the entries that are added after the march (a
-    // cluster's CTA has a loop with and one without them: 3 % on small grids; a
-    // band asks: two loops spilled)
-    auto steps = [&](auto points) {
-      constexpr bool POINTS = decltype(points)::value;
-      int slot_new = ((a.lev0 + a.dir) % a.nslots + a.nslots) % a.nslots;
-      float* glev = ring + (long long)slot_new * a.L.field;  // the new level's field
-      const int kfrom = a.store_all ? 0 : a.nsteps - 2;      // levels from this step on go to their ring slots
-      for (int step = 0, cur = 0; step < a.nsteps; ++step, cur ^= 1) {
-        const int lcur = a.lev0 + step * a.dir;
-        const uint32_t tag = tagb + (uint32_t)step;
-        // values that the next step injects (loaded now, put in place when this step ends)
-        float pv[PER];
-        if (ni > 0 && step + 1 < a.nsteps) {
+    int slot_new = ((a.lev0 + a.dir) % a.nslots + a.nslots) % a.nslots;
+    float* glev = ring + (long long)slot_new * a.L.field;  // the new level's field
+    const int kfrom = a.store_all ? 0 : a.nsteps - 2;      // levels from this step on go to their ring slots
+    for (int step = 0, cur = 0; step < a.nsteps; ++step, cur ^= 1) {
+      const int lcur = a.lev0 + step * a.dir;
+      const uint32_t tag = tagb + (uint32_t)step;
+      // values that the next step injects (loaded now, put in place when this step ends)
+      float pv[PER];
+      if (ni > 0 && step + 1 < a.nsteps) {
 #pragma unroll
-          for (int q = 0; q < PER; ++q) pv[q] = tid + q * C2_THREADS < ni ? entry(tid + q * C2_THREADS, lcur + 2 * a.dir) : 0.f;
-        }
-        // the current level is complete: its receivers (the first level of a
-        // launch was sampled by the launch before)
-        if (ns > 0 && step > 0) sample(lcur, cur ? U1 : U0);
-        if (!BAND) {
-          __syncwarp();
-          cluster_wait();  // the level's edge rows are complete in every band
-        }
-        const bool keep = step >= kfrom;
-        const uint32_t nd = cur ? 0u - lbytes : lbytes;  // from the current level to the new one
-        // low parts of the value at shared address x: at eoff + x / 2 in the current level, at neff + x / 2 in the new one
-        const uint32_t eoff = cur ? sE0 + ebytes - (sU0 + lbytes) / 2u : sE0 - sU0 / 2u;
-        const uint32_t neff = cur ? sE0 - sU0 / 2u : sE0 + ebytes - (sU0 + lbytes) / 2u;
-        for (int un = tid; un < units; un += C2_THREADS) {
-          {
-            int4 A;
-            int cul = 0;  // LEAN: the column
-            if (LEAN) {
-              const int ch = un / nx4, first = ch * N;
-              cul = un - ch * nx4;
-              A = make_int4((first * sx + 4 + 4 * cul) * 4, (z0 + H + first) * px + HX + 4 * cul, 0,
-                            (first < nrow ? F_ON : 0) | (first + N <= nrow ? F_FULL : 0) | first << 8);
+        for (int q = 0; q < PER; ++q) pv[q] = tid + q * C2_THREADS < ni ? entry(tid + q * C2_THREADS, lcur + 2 * a.dir) : 0.f;
+      }
+      // the current level is complete: its receivers (the first level of a
+      // launch was sampled by the launch before)
+      if (ns > 0 && step > 0) sample(lcur, cur ? U1 : U0);
+      if (!BAND) {
+        __syncwarp();
+        cluster_wait();  // the level's edge rows are complete in every band
+      }
+      const bool keep = step >= kfrom;
+      const uint32_t nd = cur ? 0u - lbytes : lbytes;  // from the current level to the new one
+      // low parts of the value at shared address x: at eoff + x / 2 in the current level, at neff + x / 2 in the new one
+      const uint32_t eoff = cur ? sE0 + ebytes - (sU0 + lbytes) / 2u : sE0 - sU0 / 2u;
+      const uint32_t neff = cur ? sE0 - sU0 / 2u : sE0 + ebytes - (sU0 + lbytes) / 2u;
+      for (int un = tid; un < units; un += C2_THREADS) {
+        // the unit's entries (bands read them after the march: a register more spills)
+        uint32_t ent = LEAN || BAND ? NONE << 16 | NONE : (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
+        {
+          int4 A;
+          int cul = 0;  // LEAN: the column
+          if (LEAN) {
+            const int ch = un / nx4, first = ch * N;
+            cul = un - ch * nx4;
+            A = make_int4((first * sx + 4 + 4 * cul) * 4, (z0 + H + first) * px + HX + 4 * cul, 0,
+                          (first < nrow ? F_ON : 0) | (first + N <= nrow ? F_FULL : 0) | first << 8);
+          } else {
+            A = ldsi4(sA + (uint32_t)un * 16u);
+          }
+          const int f = A.w;
+          if (!(f & F_ON)) continue;
+          const int ds = f & F_UP ? -rs : rs, gd = f & F_UP ? -px : px, cd = (f & F_UP ? -nx4 : nx4) * 16;
+          uint32_t ua = sU0 + (cur ? lbytes : 0u) + (uint32_t)A.x;
+          // c2 of the unit's rows, in shared or in global memory (zero past the grid: padding)
+          uint32_t c2a = sC2 + (uint32_t)A.z;
+          int go = A.y;  // the row's place in a field
+          auto ld_c2 = [&](int x) { return C2S ? lds4(c2a) : __ldg(reinterpret_cast<const float4*>(a.c2 + x)); };
+          // clusters: row r, in the band or an edge row (zero outside the grid)
+          auto ld_any = [&](int r, uint32_t x, float4& u, uint2& e) {
+            if (r >= 0 && r < rpc) {
+              u = lds4(x);
+              if (COMP) e = lds2(eoff + x / 2u);
             } else {
-              A = ldsi4(sA + (uint32_t)un * 16u);
+              const int i = cur * 2 * R + (r < 0 ? r + R : r - rpc + R);
+              const uint32_t co = (uint32_t)(4 + 4 * (LEAN ? cul : ldsi(sB + (uint32_t)un * 16u + 12u)));
+              u = ldc4(tab[i] + co * 4u);
+              if (COMP) e = ldc2(tab[4 * R + i] + co * 2u);
             }
-            const int f = A.w;
-            if (!(f & F_ON)) continue;
-            const int ds = f & F_UP ? -rs : rs, gd = f & F_UP ? -px : px, cd = (f & F_UP ? -nx4 : nx4) * 16;
-            uint32_t ua = sU0 + (cur ? lbytes : 0u) + (uint32_t)A.x;
-            // c2 of the unit's rows, in shared or in global memory (zero past the grid: padding)
-            uint32_t c2a = sC2 + (uint32_t)A.z;
-            int go = A.y;  // the row's place in a field
-            auto ld_c2 = [&](int x) { return C2S ? lds4(c2a) : __ldg(reinterpret_cast<const float4*>(a.c2 + x)); };
-            // clusters: row r, in the band or an edge row (zero outside the grid)
-            auto ld_any = [&](int r, uint32_t x, float4& u, uint2& e) {
-              if (r >= 0 && r < rpc) {
-                u = lds4(x);
-                if (COMP) e = lds2(eoff + x / 2u);
-              } else {
-                const int i = cur * 2 * R + (r < 0 ? r + R : r - rpc + R);
-                const uint32_t co = (uint32_t)(4 + 4 * (LEAN ? cul : ldsi(sB + (uint32_t)un * 16u + 12u)));
-                u = ldc4(tab[i] + co * 4u);
-                if (COMP) e = ldc2(tab[4 * R + i] + co * 2u);
-              }
-            };
-            const int start = f >> 8, d = f & F_UP ? -1 : 1;
-            constexpr int BL = N % 4 == 0 ? 4 : N;  // rows of an unrolled block
-            float4 u[BL + 2 * R], cqn = ld_c2(go);
-            constexpr bool EQ = COMP && !BAND;  // low parts queued too (bands: read for every row, a second queue spilled)
-            uint2 e[EQ ? BL + 2 * R : 1];
-            uint32_t ha = ua - (uint32_t)(R * ds);  // a row's address as it enters the queue
+          };
+          const int start = f >> 8, d = f & F_UP ? -1 : 1;
+          constexpr int BL = N % 4 == 0 ? 4 : N;  // rows of an unrolled block
+          float4 u[BL + 2 * R], cqn = ld_c2(go);
+          constexpr bool EQ = COMP && !BAND;  // low parts queued too (bands: read for every row, a second queue spilled)
+          uint2 e[EQ ? BL + 2 * R : 1];
+          uint32_t ha = ua - (uint32_t)(R * ds);  // a row's address as it enters the queue
 #pragma unroll
-            for (int i = 0; i < 2 * R; ++i) {
-              if (!BAND) {
-                ld_any(start + d * (i - R), ha, u[i], e[EQ ? i : 0]);
-              } else if (i >= R || !(f & (F_NB | F_OUT))) {  // N >= R: the rows of the march, or those of the chunk behind
-                u[i] = lds4(ha);
+          for (int i = 0; i < 2 * R; ++i) {
+            if (!BAND) {
+              ld_any(start + d * (i - R), ha, u[i], e[EQ ? i : 0]);
+            } else if (i >= R || !(f & (F_NB | F_OUT))) {  // N >= R: the rows of the march, or those of the chunk behind
+              u[i] = lds4(ha);
+            }
+            ha += (uint32_t)ds;
+          }
+          if (BAND && f & F_NB) {
+            const uint32_t o = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 4u) + (tag & 1u) * epar, st = f & F_UP ? erow : 0u - erow;
+            constexpr int G = COMP ? 2 : R;  // rows asked for at once
+#pragma unroll
+            for (int k0 = 0; k0 < R; k0 += G) {
+              if (!ahead) {
+#pragma unroll
+                for (int k = k0; k < k0 + G; ++k) ask(k, o + (uint32_t)k * st);
+              }
+#pragma unroll
+              for (int k = k0; k < k0 + G; ++k) {
+                uint4& x = wa[BAND ? k : 0];
+                uint4& y = wb[BAND ? k : 0];
+                uint4& z = wc[BAND && COMP ? k : 0];
+                settle(o + (uint32_t)k * st, x, y, z, tag);
+                u[R - 1 - k] = make_float4(__uint_as_float(x.x), __uint_as_float(x.z), __uint_as_float(y.x), __uint_as_float(y.z));
+                if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(z.x, z.z));
+              }
+            }
+          } else if (BAND && f & F_OUT) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+              u[R - 1 - k] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(0u, 0u));
+            }
+          }
+          const bool pub = BAND && f & F_PUB && step + 1 < a.nsteps;
+          uint32_t w = pub ? (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar : 0u;
+          const uint32_t wd = f & F_UP ? 0u - erow : erow;
+#pragma unroll 1
+          for (int b = 0; b < N / BL; ++b) {
+#pragma unroll
+            for (int jj = 0; jj < BL; ++jj) {
+              if (LEAN && start + jj >= rpc) break;  // the last chunk's rows
+              // the row R beyond this one completes the queue (bands: a row of the next chunk at most)
+              if (BAND) {
+                u[jj + 2 * R] = lds4(ha);
+              } else {
+                ld_any(start + d * (b * BL + jj + R), ha, u[jj + 2 * R], e[EQ ? jj + 2 * R : 0]);
               }
               ha += (uint32_t)ds;
-            }
-            if (BAND && f & F_NB) {
-              const uint32_t o = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 4u) + (tag & 1u) * epar, st = f & F_UP ? erow : 0u - erow;
-              constexpr int G = COMP ? 2 : R;  // rows asked for at once
+              const float4 cq = cqn;
+              c2a += (uint32_t)cd;
+              if (jj + 1 < BL || b + 1 < N / BL) cqn = ld_c2(go + gd);
+              const uint32_t na = ua + nd;
+              float o[4], en[4] = {0.f, 0.f, 0.f, 0.f};
+              float4 c1;
+              float2 s2[2];
+              auto low = [&](int k) {
+                if constexpr (EQ) return e[jj + R + k];
+                else return lds2(eoff + ua / 2u + (uint32_t)(k * ds / 2));
+              };
+              row4<R, MODE>(a.W, u + jj, low, cq, ua, na, eoff, neff, o, en, c1, s2);
+              if (DAMP) {
+                const int dz = nz - 1 - (z0 + start + d * (b * BL + jj)), cu = ldsi(sB + (uint32_t)un * 16u + 12u);
+                if (min(min(4 * cu, nx - 4 - 4 * cu), dz) < a.W.sw) {
 #pragma unroll
-              for (int k0 = 0; k0 < R; k0 += G) {
-                if (!ahead) {
-#pragma unroll
-                  for (int k = k0; k < k0 + G; ++k) ask(k, o + (uint32_t)k * st);
-                }
-#pragma unroll
-                for (int k = k0; k < k0 + G; ++k) {
-                  uint4& x = wa[BAND ? k : 0];
-                  uint4& y = wb[BAND ? k : 0];
-                  uint4& z = wc[BAND && COMP ? k : 0];
-                  settle(o + (uint32_t)k * st, x, y, z, tag);
-                  u[R - 1 - k] = make_float4(__uint_as_float(x.x), __uint_as_float(x.z), __uint_as_float(y.x), __uint_as_float(y.z));
-                  if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(z.x, z.z));
-                }
-              }
-            } else if (BAND && f & F_OUT) {
-#pragma unroll
-              for (int k = 0; k < R; ++k) {
-                u[R - 1 - k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (COMP) sts2(eoff + ua / 2u - (uint32_t)((k + 1) * (ds / 2)), make_uint2(0u, 0u));
-              }
-            }
-            const bool pub = BAND && f & F_PUB && step + 1 < a.nsteps;
-            uint32_t w = pub ? (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar : 0u;
-            const uint32_t wd = f & F_UP ? 0u - erow : erow;
-#pragma unroll 1
-            for (int b = 0; b < N / BL; ++b) {
-#pragma unroll
-              for (int jj = 0; jj < BL; ++jj) {
-                if (LEAN && start + jj >= rpc) break;  // the last chunk's rows
-                // the row R beyond this one completes the queue (bands: a row of the next chunk at most)
-                if (BAND) {
-                  u[jj + 2 * R] = lds4(ha);
-                } else {
-                  ld_any(start + d * (b * BL + jj + R), ha, u[jj + 2 * R], e[EQ ? jj + 2 * R : 0]);
-                }
-                ha += (uint32_t)ds;
-                const float4 cq = cqn;
-                c2a += (uint32_t)cd;
-                if (jj + 1 < BL || b + 1 < N / BL) cqn = ld_c2(go + gd);
-                const uint32_t na = ua + nd;
-                float o[4], en[4] = {0.f, 0.f, 0.f, 0.f};
-                float4 c1;
-                float2 s2[2];
-                auto low = [&](int k) {
-                  if constexpr (EQ) return e[jj + R + k];
-                  else return lds2(eoff + ua / 2u + (uint32_t)(k * ds / 2));
-                };
-                row4<R, MODE>(a.W, u + jj, low, cq, ua, na, eoff, neff, o, en, c1, s2);
-                if (DAMP) {
-                  const int dz = nz - 1 - (z0 + start + d * (b * BL + jj)), cu = ldsi(sB + (uint32_t)un * 16u + 12u);
-                  if (min(min(4 * cu, nx - 4 - 4 * cu), dz) < a.W.sw) {
-#pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                      const int dd = min(min(4 * cu + p, nx - 1 - (4 * cu + p)), dz);
-                      const float2 ai = dmp[dd >= 0 && dd < a.W.sw ? dd : a.W.sw];
-                      // tp_stencil.cu's epilogue; a = 0 (outside the layer) gives the undamped value
-                      o[p] = quotient(fmaf(comp4(cq, p), p & 1 ? s2[p / 2].y : s2[p / 2].x,
-                                           fmaf(-(1.0f - ai.x), comp4(c1, p), 2.0f * comp4(u[jj + R], p))),
-                                      1.0f + ai.x, ai.y);
-                    }
+                  for (int p = 0; p < 4; ++p) {
+                    const int dd = min(min(4 * cu + p, nx - 1 - (4 * cu + p)), dz);
+                    const float2 ai = dmp[dd >= 0 && dd < a.W.sw ? dd : a.W.sw];
+                    // tp_stencil.cu's epilogue; a = 0 (outside the layer) gives the undamped value
+                    o[p] = quotient(fmaf(comp4(cq, p), p & 1 ? s2[p / 2].y : s2[p / 2].x,
+                                         fmaf(-(1.0f - ai.x), comp4(c1, p), 2.0f * comp4(u[jj + R], p))),
+                                    1.0f + ai.x, ai.y);
                   }
                 }
-                // the new value over the previous level (own points: no other thread reads them in this step)
-                const float4 ov = make_float4(o[0], o[1], o[2], o[3]);
-                const uint2 ev = COMP ? to_bf4(make_float4(en[0], en[1], en[2], en[3])) : make_uint2(0u, 0u);
-                sts4(na, ov);
-                if (COMP) sts2(neff + na / 2u, ev);
-                if (keep && (f & F_FULL || start + d * (b * BL + jj) < nrow)) *reinterpret_cast<float4*>(glev + go) = ov;
-                go += gd;
-                ua += (uint32_t)ds;
-                if (BAND && jj < R && b == 0 && pub) {
-                  publish(w, ov, ev, tag + 1);
-                  w += wd;
-                }
               }
-              if (N > BL) {
-#pragma unroll
-                for (int i = 0; i < 2 * R; ++i) {
-                  u[i] = u[i + BL];
-                  if (EQ) e[EQ ? i : 0] = e[EQ ? i + BL : 0];
-                }
+              // the new value over the previous level (own points: no other thread reads them in this step)
+              const float4 ov = make_float4(o[0], o[1], o[2], o[3]);
+              const uint2 ev = COMP ? to_bf4(make_float4(en[0], en[1], en[2], en[3])) : make_uint2(0u, 0u);
+              sts4(na, ov);
+              if (COMP) sts2(neff + na / 2u, ev);
+              if (keep && (f & F_FULL || start + d * (b * BL + jj) < nrow)) *reinterpret_cast<float4*>(glev + go) = ov;
+              go += gd;
+              ua += (uint32_t)ds;
+              if (BAND && jj < R && b == 0 && pub) {
+                publish(w, ov, ev, tag + 1);
+                w += wd;
               }
             }
-          }
-          // entries at this unit's points, added to the values just stored
-          const uint32_t ent = LEAN ? NONE << 16 | NONE : (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
-          if (ent != (NONE << 16 | NONE)) {
-            const int f = ldsi(sA + (uint32_t)un * 16u + 12u), start = f >> 8, d = f & F_UP ? -1 : 1;
-            const int cu = ldsi(sB + (uint32_t)un * 16u + 12u);
-            const float* v = ival + (step & 1) * vstep;
-            float* const Un = cur ? U0 : U1;
-            __nv_bfloat16* const En = cur ? E0 : E1;
-            if (ent >> 16 != NONE) {  // a line: one row, one entry per point at most
-              const int r = start + d * (int)(ent >> 16), l = r * sx + 4 + 4 * cu;
-              const ushort4 k = uline[un];
-              const float val[4] = {v[k.x], v[k.y], v[k.z], v[k.w]};
-              float4 x = *reinterpret_cast<const float4*>(Un + l);
-              float o[4] = {x.x, x.y, x.z, x.w};
-              if (COMP) {
-                const float4 ee = bf4(*reinterpret_cast<const uint2*>(En + l));
-                float eo[4] = {ee.x, ee.y, ee.z, ee.w};
+            if (N > BL) {
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                  float err;
-                  o[p] = two_sum(o[p], val[p], &err);
-                  eo[p] += err;
-                }
-                *reinterpret_cast<uint2*>(En + l) = to_bf4(make_float4(eo[0], eo[1], eo[2], eo[3]));
-              } else {
-#pragma unroll
-                for (int p = 0; p < 4; ++p) o[p] = o[p] + val[p];
-              }
-              x = make_float4(o[0], o[1], o[2], o[3]);
-              *reinterpret_cast<float4*>(Un + l) = x;
-              if (keep) *reinterpret_cast<float4*>(glev + (long long)(z0 + H + r) * px + HX + 4 * cu) = x;
-            }
-            // a chain: by node, a node's entries in index order
-            for (uint32_t i = BAND ? ent & NONE : NONE; i != NONE;) {
-              const uint32_t l = il[i] >> 16;
-              float x = Un[l], xe = COMP ? __bfloat162float(En[l]) : 0.f;
-              for (; i != NONE && il[i] >> 16 == l; i = nxt[i]) {
-                if (COMP) {
-                  float err;
-                  x = two_sum(x, v[i], &err);
-                  xe += err;
-                } else {
-                  x = x + v[i];
-                }
-              }
-              Un[l] = x;
-              if (COMP) En[l] = __float2bfloat16(xe);
-              const int r = (int)l / sx;
-              if (keep) glev[(long long)(z0 + H + r) * px + HX + ((int)l - r * sx - 4)] = x;
-            }
-          }
-          if (BAND && ent != (NONE << 16 | NONE) && step + 1 < a.nsteps) {
-            const int4 A = ldsi4(sA + (uint32_t)un * 16u);
-            if (A.w & F_LATE) {
-              const uint32_t w = (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar;
-              for (int j = 0; j < R; ++j) {
-                const uint32_t x = sU0 + (cur ? 0u : lbytes) + (uint32_t)(A.x + j * (A.w & F_UP ? -rs : rs));
-                publish(w + (uint32_t)(j * (A.w & F_UP ? -(int)erow : (int)erow)), lds4(x),
-                        COMP ? lds2(neff + x / 2u) : make_uint2(0u, 0u), tag + 1);
+              for (int i = 0; i < 2 * R; ++i) {
+                u[i] = u[i + BL];
+                if (EQ) e[EQ ? i : 0] = e[EQ ? i + BL : 0];
               }
             }
           }
         }
-        if (POINTS && !WALK && (!BAND || ldsi(sLead))) {  // the other units' entries: a thread adds all of a node's, in order
-          __syncthreads();
+        // entries at this unit's points, added to the values just stored
+        if (BAND) ent = (uint32_t)ldsi(sB + (uint32_t)un * 16u + 8u);
+        if (ent != (NONE << 16 | NONE)) {
+          const int f = ldsi(sA + (uint32_t)un * 16u + 12u), start = f >> 8, d = f & F_UP ? -1 : 1;
+          const int cu = ldsi(sB + (uint32_t)un * 16u + 12u);
           const float* v = ival + (step & 1) * vstep;
           float* const Un = cur ? U0 : U1;
           __nv_bfloat16* const En = cur ? E0 : E1;
-          for (int i = tid; i < ni; i += C2_THREADS) {
-            const uint32_t e = il[i], l = e >> 16;
-            if (!(e & LEAD)) continue;
-            const int n = nxt[i];
+          if (ent >> 16 != NONE) {  // a line: one row, one entry per point at most
+            const int r = start + d * (int)(ent >> 16), l = r * sx + 4 + 4 * cu;
+            const ushort4 k = uline[un];
+            const float val[4] = {v[k.x], v[k.y], v[k.z], v[k.w]};
+            float4 x = *reinterpret_cast<const float4*>(Un + l);
+            float o[4] = {x.x, x.y, x.z, x.w};
+            if (COMP) {
+              const float4 ee = bf4(*reinterpret_cast<const uint2*>(En + l));
+              float eo[4] = {ee.x, ee.y, ee.z, ee.w};
+#pragma unroll
+              for (int p = 0; p < 4; ++p) {
+                float err;
+                o[p] = two_sum(o[p], val[p], &err);
+                eo[p] += err;
+              }
+              *reinterpret_cast<uint2*>(En + l) = to_bf4(make_float4(eo[0], eo[1], eo[2], eo[3]));
+            } else {
+#pragma unroll
+              for (int p = 0; p < 4; ++p) o[p] = o[p] + val[p];
+            }
+            x = make_float4(o[0], o[1], o[2], o[3]);
+            *reinterpret_cast<float4*>(Un + l) = x;
+            if (keep) *reinterpret_cast<float4*>(glev + (long long)(z0 + H + r) * px + HX + 4 * cu) = x;
+          }
+          // a chain: by node, a node's entries in index order
+          for (uint32_t i = LEAN ? NONE : ent & NONE; i != NONE;) {
+            const uint32_t l = il[i] >> 16;
             float x = Un[l], xe = COMP ? __bfloat162float(En[l]) : 0.f;
-#pragma unroll 4
-            for (int k = 0; k < n; ++k) {
+            auto add = [&](float val) {
               if (COMP) {
                 float err;
-                x = two_sum(x, v[i + k], &err);
+                x = two_sum(x, val, &err);
                 xe += err;
               } else {
-                x = x + v[i + k];
+                x = x + val;
               }
+            };
+            if (WALK) {
+              const int n = il[i] & MANY ? nxt[i] : 1;
+#pragma unroll 4
+              for (int k = 0; k < n; ++k) add(v[i + k]);
+              i = nxt[i + n - 1];
+            } else {  // (as above it spills)
+              for (; i != NONE && il[i] >> 16 == l; i = nxt[i]) add(v[i]);
             }
             Un[l] = x;
             if (COMP) En[l] = __float2bfloat16(xe);
@@ -934,25 +907,60 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
             if (keep) glev[(long long)(z0 + H + r) * px + HX + ((int)l - r * sx - 4)] = x;
           }
         }
-        if (ni > 0 && step + 1 < a.nsteps) {
-#pragma unroll
-          for (int q = 0; q < PER; ++q)
-            if (tid + q * C2_THREADS < ni) ival[((step + 1) & 1) * vstep + tid + q * C2_THREADS] = pv[q];
+        if (BAND && ent != (NONE << 16 | NONE) && step + 1 < a.nsteps) {
+          const int4 A = ldsi4(sA + (uint32_t)un * 16u);
+          if (A.w & F_LATE) {
+            const uint32_t w = (uint32_t)ldsi(sB + (uint32_t)un * 16u) + epar - (tag & 1u) * epar;
+            for (int j = 0; j < R; ++j) {
+              const uint32_t x = sU0 + (cur ? 0u : lbytes) + (uint32_t)(A.x + j * (A.w & F_UP ? -rs : rs));
+              publish(w + (uint32_t)(j * (A.w & F_UP ? -(int)erow : (int)erow)), lds4(x),
+                      COMP ? lds2(neff + x / 2u) : make_uint2(0u, 0u), tag + 1);
+            }
+          }
         }
-        // the words of the next level's edge rows, on their way while the CTA gathers
-        if (step + 1 < a.nsteps) ask_ahead(tag + 1);
-        slot_new += a.dir;
-        glev += a.dir * a.L.field;
-        if (slot_new == a.nslots || slot_new < 0) {
-          glev -= a.dir * (long long)a.nslots * a.L.field;
-          slot_new = slot_new < 0 ? a.nslots - 1 : 0;
-        }
-        __syncthreads();  // the new level is complete in this band
-        if (!BAND) cluster_arrive();
       }
-    };
-    if (BAND || cnt[3]) steps(std::true_type{});
-    else steps(std::false_type{});
+      if (!WALK && ldsi(sLead)) {  // the other units' entries: a thread adds all of a node's, in order
+        __syncthreads();
+        const float* v = ival + (step & 1) * vstep;
+        float* const Un = cur ? U0 : U1;
+        __nv_bfloat16* const En = cur ? E0 : E1;
+        for (int i = tid; i < ni; i += C2_THREADS) {
+          const uint32_t e = il[i], l = e >> 16;
+          if (!(e & LEAD)) continue;
+          const int n = nxt[i];
+          float x = Un[l], xe = COMP ? __bfloat162float(En[l]) : 0.f;
+#pragma unroll 4
+          for (int k = 0; k < n; ++k) {
+            if (COMP) {
+              float err;
+              x = two_sum(x, v[i + k], &err);
+              xe += err;
+            } else {
+              x = x + v[i + k];
+            }
+          }
+          Un[l] = x;
+          if (COMP) En[l] = __float2bfloat16(xe);
+          const int r = (int)l / sx;
+          if (keep) glev[(long long)(z0 + H + r) * px + HX + ((int)l - r * sx - 4)] = x;
+        }
+      }
+      if (ni > 0 && step + 1 < a.nsteps) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q)
+          if (tid + q * C2_THREADS < ni) ival[((step + 1) & 1) * vstep + tid + q * C2_THREADS] = pv[q];
+      }
+      // the words of the next level's edge rows, on their way while the CTA gathers
+      if (step + 1 < a.nsteps) ask_ahead(tag + 1);
+      slot_new += a.dir;
+      glev += a.dir * a.L.field;
+      if (slot_new == a.nslots || slot_new < 0) {
+        glev -= a.dir * (long long)a.nslots * a.L.field;
+        slot_new = slot_new < 0 ? a.nslots - 1 : 0;
+      }
+      __syncthreads();  // the new level is complete in this band
+      if (!BAND) cluster_arrive();
+    }
     // the last level's receivers, and the low parts of the last two levels
     // (the next launch starts from them)
     const int lfin = a.lev0 + a.nsteps * a.dir;
