@@ -44,9 +44,9 @@
 // measurements.
 // Measured per step on GB300 (forward calls of 1500 and 300 levels, their
 // difference), before (clusters only, one CTA of 16 warps with guarded rows) and
-// now: 601 x 201, 16 shots, order 8: levels 6.1 -> 3.6 us, compensated 13.2 ->
-// 7.8 us; 801 x 301, 8 shots: 6.4 -> 3.6, 19.7 -> 8.2 us; 101 x 101, one shot,
-// order 4: 1.7 -> 1.25 us; an absorbing layer (601 x 201, 4 shots, then two
+// now: 601 x 201, 16 shots, order 8: levels 6.1 -> 3.7 us, compensated 13.2 ->
+// 7.9 us; 801 x 301, 8 shots: 6.4 -> 3.7, 19.7 -> 8.2 us; 101 x 101, one shot,
+// order 4: 1.7 -> 1.2 us; an absorbing layer (601 x 201, 4 shots, then two
 // launches per step) 31 -> 4.2 us.  Bound by the shared memory
 // pipe (32 wavefronts per 128 points of the levels form: the row and its
 // neighbours, c2, the previous and the new level, the ring) and by issue.
@@ -312,8 +312,8 @@ __device__ __forceinline__ void row4(const Weights& W, const float4* u, Low low,
 // LEAN (clusters without c2 in shared memory, for wide grids): the levels alone
 // fill the shared memory.  c2 comes from global memory, nothing is kept per
 // unit, all entries are added after the march, and the last chunk of a band
-// has as many rows as are left.  Compensated step, order 8: 1800 x 100 8.6 us,
-// 2001 x 101 x 8 shots 10.9 us (8.3 and 17.1 us when a cluster kept c2 in global
+// has as many rows as are left.  Compensated step, order 8: 1800 x 100 8.4 us,
+// 2001 x 101 x 8 shots 10.6 us (8.3 and 17.1 us when a cluster kept c2 in global
 // memory and guarded every row).
 template <int R, int MODE, bool BAND, int N, bool C2S>
 __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(C2_THREADS, 1) sweep2d_shots(C2Args a) {
   // walked along nxt when the unit is marched; the others are added after the
   // march, where an entry with LEAD stands for the nxt entries of its node from
   // it on.  (WALK: so does one with MANY, and the last of them leads on.)  Step at
-  // 401 x 401 with 1024 receivers at a node 9.8 us, in a patch of 32 x 32 5.7 us,
+  // 401 x 401 with 1024 receivers at a node 9.7 us, in a patch of 32 x 32 5.6 us,
   // along a borehole 4.4 us, in a row 3.5 us (14 ms, 43, 7.5 and 4.0 us when the
   // unit's thread walked the chain once for every entry).
   // Per unit, read where it is used (kept in registers, it spilled):
@@ -1118,7 +1118,7 @@ int c2_sms() {
 
 // The best split into bands of one cooperative grid (C = 0: none fits), by rank;
 // fit (may be null): with a fifth of the estimate, which tells the splits at the
-// floor apart (601 x 201: 26 bands of 8 rows 3.2 us, 13 of 16 4.1).  With a layer,
+// floor apart (601 x 201: 26 bands of 8 rows 3.4 us, 13 of 16 4.1).  With a layer,
 // whose marches are longer, both by the estimate (order 4, 601 x 201 x 16: 5.3 us,
 // by rank 5.9).
 C2Plan c2_bands(const Layout& L, int R, int mode, int sw, int nshots, int capi, int caps, C2Plan* fit) {
@@ -1181,7 +1181,7 @@ int c2_max_clusters(int C, size_t smem) {
 // march; another one (clusters of four rows and lean ones included) where the
 // fitted estimate gives it 10 % less.  Over the 480 grids no split chosen so is
 // more than 3 % slower than the one by rank alone and 52 are faster by more (1500 x
-// 60 2.7 us a step instead of 5.0, 601 x 201 3.2 instead of 4.3, 2000 x 64 x 2 3.3
+// 60 2.7 us a step instead of 5.0, 601 x 201 3.4 instead of 4.3, 2000 x 64 x 2 3.3
 // instead of 4.4); by the estimate alone 13 and 104.  The chosen split takes on
 // average 3.0 % longer than the best measured one (by rank 5.0 %).
 template <int R, int MODE>
